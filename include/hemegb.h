@@ -121,18 +121,15 @@ typedef struct {
                                      the gathers and the scatter, packed rest values, the
                                      even step on vector pairs (sites_per_thread 2);
                                  7 = 6 with L2 256-byte prefetch hints on the loads;
-                                 8, 9, 10, 11 = 3, 5, 6, 7 reading the run-encoded
-                                     neighbour table (hg_domain_runs) instead of the
-                                     18 table rows; a launch over a domain without
-                                     one runs 3, 5, 6, 7; same shapes as 3, 5, 6, 7;
-                                 12 = 8 for AA (1 or 2 sites per thread) with the odd
-                                     step's 18 entries stashed in shared memory
-                                     across the collision instead of decoded twice;
-                                 13 = 8 (2 or 4 sites per thread) with every site's
-                                     link word loaded, and its run row prefetched,
-                                     before the first site's gathers;
-                                 14 = 10 with the stash of 12 (AA, 2 sites per
-                                     thread) */
+                                 8..14 = one kernel that reads the run-encoded neighbour
+                                     table (hg_domain_runs) instead of the 18 table
+                                     rows, in a launch shape of its own; a launch over
+                                     a domain without a run encoding runs variant 3
+                                     (8, 12, 13), 5 (9), 6 (10, 14) or 7 (11) in the
+                                     shape given.  The shapes accepted with them: any
+                                     (8); those of 5 (9), of 6 (10, 11, 14); 1 or 2
+                                     sites per thread, AA (12); 2 or 4 sites per
+                                     thread (13) */
     void *stream;             /* cudaStream_t to order work on; NULL = a stream the context creates */
     hg_alloc_fn alloc;        /* NULL = cudaMalloc */
     hg_free_fn free;          /* NULL = cudaFree */

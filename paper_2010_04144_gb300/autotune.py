@@ -26,11 +26,9 @@ DEFAULT_CANDIDATES = (
     (256, 1, 3), (128, 1, 3), (256, 2, 3), (128, 2, 3), (512, 2, 3), (128, 4, 3), (256, 4, 3),
     (128, 2, 5), (256, 2, 5), (512, 2, 5),  # variant 5: A/B with 16-bit storage only
     (128, 2, 6), (256, 2, 6), (256, 2, 7), (512, 2, 7),  # variants 6, 7: AA on site pairs
-    # 8..11: 3, 5, 6, 7 reading the run-encoded neighbour table
-    (256, 1, 8), (128, 2, 8), (256, 2, 8), (128, 2, 9), (256, 2, 9), (128, 2, 10), (256, 2, 10), (256, 2, 11),
-    (256, 1, 12), (128, 1, 12), (128, 2, 12),  # 12: AA, run-encoded, odd-step entries stashed
-    (128, 2, 13), (256, 2, 13), (128, 4, 13),  # 13: run-encoded, link words hoisted
-    (128, 2, 14), (256, 2, 14),  # 14: AA pairs even, run-encoded odd with the stash
+    # 8..14: the run-encoded neighbour table, one kernel in a shape of its own; on domains
+    # without one they are 3, 5, 6 and 7 in the shape given
+    (256, 1, 8), (256, 2, 9), (256, 2, 10), (256, 2, 11), (128, 1, 12), (128, 2, 13), (128, 2, 14),
 )
 # Variant 4 (staged AA odd-step stores) is measured slower than variant 1 on
 # every workload tried; it stays available through Context.set_launch.

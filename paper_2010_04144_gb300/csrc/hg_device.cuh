@@ -96,118 +96,159 @@ template <int B, int E, typename F> __device__ __forceinline__ void unroll(F &&f
 // in the collision variable.  Scaled storage (h = f~/w) drops the w_I factors
 // (w_I = w_opp(I)); its velocity coefficients are stored divided by w_I.
 template <int I, bool SC>
-__device__ __forceinline__ float iolet_rule(const DomDev &D, int k, int slot, float raw) {
-    const float val = D.bcv[k];
+__device__ __forceinline__ float iolet_rule(const DomDev &D, const float *bcv, int k, int slot, float raw) {
+    const float val = bcv[k];
     if (D.io_kind[k] == 0) return -raw + (SC ? 2.0f * val : mulw<I>(2.0f * val));  // anti-bounce-back
-    return raw + val * D.coef[(int64_t)slot * 18 + (I - 1)];              // moving wall
+    return __fmaf_rn(val, D.coef[(int64_t)slot * 18 + (I - 1)], raw);       // moving wall
 }
 
 // LBGK collision in deviation form, in place on g[19]; returns (drho, u).
-// Every product and sum is written with explicit rounding intrinsics (__fmul_rn,
-// __fadd_rn, __fmaf_rn), so the compiler cannot contract them differently in the
-// different kernels that inline this: all variants produce the same bits.
+// Every product and sum is written with explicit rounding intrinsics, so the compiler
+// cannot contract them differently in the different kernels that inline this: all
+// variants produce the same bits.
 #define HG_MUL __fmul_rn
 #define HG_ADD __fadd_rn
 #define HG_SUB __fsub_rn
 #define HG_FMA __fmaf_rn
 
-// SC: the scaled variable h = f~/w (16-bit storage), whose equilibrium carries no
-// weight; otherwise f~, whose equilibrium is w times that (split-weight products).
-template <bool SC>
-__device__ __forceinline__ void relax_pairs(float g[19], float omega, float base, float rho,
-                                            float ux, float uy, float uz) {
-    const float r45 = HG_MUL(4.5f, rho), r3 = HG_MUL(3.0f, rho);
-    auto pair = [&](auto ia, int b, float cu) {
+// Two FP32 values (the same quantity of two sites) in one 64-bit register pair.  sm_103a
+// adds, multiplies and fuses both with one instruction, each half rounded exactly as the
+// scalar instruction rounds it.  The 16-bit kernels and the FP32 kernels with a decoded
+// table were bound by instruction issue, and the collision is half of their instructions.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pk2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float lo2(F2 x) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+    return a;
+}
+__device__ __forceinline__ float hi2(F2 x) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+    return b;
+}
+__device__ __forceinline__ float vadd(float a, float b) { return HG_ADD(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return HG_SUB(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return HG_MUL(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return HG_FMA(a, b, c); }
+__device__ __forceinline__ float vrcp(float a) { return __frcp_rn(a); }
+__device__ __forceinline__ F2 vadd(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vsub(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vmul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 vrcp(F2 a) { return pk2(__frcp_rn(lo2(a)), __frcp_rn(hi2(a))); }
+// A product that a following addition must not be fused with: ptxas contracts
+// mul.rn.f32x2 + add.rn.f32x2 (as it never does the scalar pair), so the packed product is
+// formed as a b + z with z = (-0, -0) that the compiler does not know (it adds nothing).
+__device__ __forceinline__ float vmul_apart(float a, float b, unsigned long long) { return HG_MUL(a, b); }
+__device__ __forceinline__ F2 vmul_apart(F2 a, F2 b, unsigned long long z) { return vfma(a, b, F2{z}); }
+template <typename V> __device__ __forceinline__ V vset(float x);
+template <> __device__ __forceinline__ float vset<float>(float x) { return x; }
+template <> __device__ __forceinline__ F2 vset<F2>(float x) { return pk2(x, x); }
+template <int I, typename V> __device__ __forceinline__ V vmulw(V x) {  // mulw<I>, see above
+    return vfma(vset<V>(W(I)), x, vmul(vset<V>(WLO(I)), x));
+}
+
+// (drho, ux, uy, uz) of one site (V = float) or two (V = F2)
+template <typename V> struct MomT {
+    V drho, ux, uy, uz;
+};
+
+// SC: the scaled variable h = f~/w (16-bit storage): its moments weight h by w, its
+// equilibrium h~eq_i = drho + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u.u) carries no weight.
+// Otherwise f~, whose equilibrium is w times that (split-weight products).
+template <bool SC, typename V>
+__device__ __forceinline__ MomT<V> collide_v(V g[19], float omega_, unsigned long long neg_zero2) {
+    V drho, jx, jy, jz;
+    const V d12 = vsub(g[1], g[2]), d34 = vsub(g[3], g[4]), d56 = vsub(g[5], g[6]);
+    const V d78 = vsub(g[7], g[8]), d910 = vsub(g[9], g[10]), d1112 = vsub(g[11], g[12]);
+    const V d1314 = vsub(g[13], g[14]), d1516 = vsub(g[15], g[16]), d1718 = vsub(g[17], g[18]);
+    if constexpr (SC) {
+        const V sa = vadd(vadd(vadd(g[1], g[2]), vadd(g[3], g[4])), vadd(g[5], g[6]));
+        const V sd = vadd(vadd(vadd(vadd(g[7], g[8]), vadd(g[9], g[10])),
+                               vadd(vadd(g[11], g[12]), vadd(g[13], g[14]))),
+                          vadd(vadd(g[15], g[16]), vadd(g[17], g[18])));
+        drho = vadd(vmulw<0>(g[0]), vadd(vmulw<1>(sa), vmulw<7>(sd)));
+        const V ex = vadd(vadd(d78, d910), vadd(d1112, d1314));
+        const V ey = vadd(vsub(d78, d910), vadd(d1516, d1718));
+        const V ez = vadd(vsub(d1112, d1314), vsub(d1516, d1718));
+        jx = vadd(vmulw<1>(d12), vmulw<7>(ex));
+        jy = vadd(vmulw<1>(d34), vmulw<7>(ey));
+        jz = vadd(vmulw<1>(d56), vmulw<7>(ez));
+    } else {
+        drho = g[0];
+#pragma unroll
+        for (int i = 1; i < 19; ++i) drho = vadd(drho, g[i]);
+        jx = vadd(vadd(vadd(d12, d78), vadd(d910, d1112)), d1314);
+        jy = vadd(vadd(vsub(vadd(d34, d78), d910), d1516), d1718);
+        jz = vsub(vadd(vsub(vadd(d56, d1112), d1314), d1516), d1718);
+    }
+    const V omega = vset<V>(omega_);
+    const V rho = vadd(vset<V>(1.0f), drho);
+    const V inv = vrcp(rho);
+    const V ux = vmul(jx, inv), uy = vmul(jy, inv), uz = vmul(jz, inv);
+    const V usq = vfma(ux, ux, vfma(uy, uy, vmul(uz, uz)));
+    const V base = vfma(vmul(vset<V>(-1.5f), rho), usq, drho);  // drho - 1.5 rho u.u
+    const V r45 = vmul(vset<V>(4.5f), rho), r3 = vmul(vset<V>(3.0f), rho);
+    if constexpr (SC) g[0] = vfma(omega, vsub(base, g[0]), g[0]);
+    else g[0] = vfma(omega, vsub(vmulw<0>(base), g[0]), g[0]);
+    auto pair = [&](auto ia, int b, V cu) {
         constexpr int a = decltype(ia)::v;
-        const float q = HG_FMA(HG_MUL(r45, cu), cu, base);    // base + 4.5 rho cu^2
-        const float c3 = HG_MUL(r3, cu);
-        const float sym = SC ? q : mulw<a>(q);
-        const float asym = SC ? c3 : mulw<a>(c3);
-        g[a] = HG_FMA(omega, HG_SUB(HG_ADD(sym, asym), g[a]), g[a]);
-        g[b] = HG_FMA(omega, HG_SUB(HG_SUB(sym, asym), g[b]), g[b]);
+        const V q = vfma(vmul(r45, cu), cu, base);    // base + 4.5 rho cu^2
+        const V c3 = vmul_apart(r3, cu, neg_zero2);
+        V sym = q, asym = c3;
+        if constexpr (!SC) {
+            sym = vmulw<a>(q);
+            asym = vmulw<a>(c3);
+        }
+        g[a] = vfma(omega, vsub(vadd(sym, asym), g[a]), g[a]);
+        g[b] = vfma(omega, vsub(vsub(sym, asym), g[b]), g[b]);
     };
     pair(IC<1>{}, 2, ux);
     pair(IC<3>{}, 4, uy);
     pair(IC<5>{}, 6, uz);
-    pair(IC<7>{}, 8, HG_ADD(ux, uy));
-    pair(IC<9>{}, 10, HG_SUB(ux, uy));
-    pair(IC<11>{}, 12, HG_ADD(ux, uz));
-    pair(IC<13>{}, 14, HG_SUB(ux, uz));
-    pair(IC<15>{}, 16, HG_ADD(uy, uz));
-    pair(IC<17>{}, 18, HG_SUB(uy, uz));
-}
-
-struct Moments {
-    float drho, ux, uy, uz, rho, base;
-};
-
-// u, rho and the equilibrium's isotropic part from drho and j.
-__device__ __forceinline__ Moments finish_moments(float drho, float jx, float jy, float jz) {
-    Moments m;
-    m.drho = drho;
-    m.rho = HG_ADD(1.0f, drho);
-    const float inv = __frcp_rn(m.rho);
-    m.ux = HG_MUL(jx, inv);
-    m.uy = HG_MUL(jy, inv);
-    m.uz = HG_MUL(jz, inv);
-    const float usq = HG_FMA(m.ux, m.ux, HG_FMA(m.uy, m.uy, HG_MUL(m.uz, m.uz)));
-    m.base = HG_FMA(HG_MUL(-1.5f, m.rho), usq, drho);       // drho - 1.5 rho u.u
-    return m;
-}
-
-__device__ __forceinline__ float4 collide(float g[19], float omega) {
-    float drho = g[0];
-#pragma unroll
-    for (int i = 1; i < 19; ++i) drho = HG_ADD(drho, g[i]);
-    const float d12 = HG_SUB(g[1], g[2]), d34 = HG_SUB(g[3], g[4]), d56 = HG_SUB(g[5], g[6]);
-    const float d78 = HG_SUB(g[7], g[8]), d910 = HG_SUB(g[9], g[10]), d1112 = HG_SUB(g[11], g[12]);
-    const float d1314 = HG_SUB(g[13], g[14]), d1516 = HG_SUB(g[15], g[16]), d1718 = HG_SUB(g[17], g[18]);
-    const float jx = HG_ADD(HG_ADD(HG_ADD(d12, d78), HG_ADD(d910, d1112)), d1314);
-    const float jy = HG_ADD(HG_ADD(HG_SUB(HG_ADD(d34, d78), d910), d1516), d1718);
-    const float jz = HG_SUB(HG_ADD(HG_SUB(HG_ADD(d56, d1112), d1314), d1516), d1718);
-    const Moments m = finish_moments(drho, jx, jy, jz);
-    g[0] = HG_FMA(omega, HG_SUB(mulw<0>(m.base), g[0]), g[0]);
-    relax_pairs<false>(g, omega, m.base, m.rho, m.ux, m.uy, m.uz);
-    return make_float4(m.drho, m.ux, m.uy, m.uz);
-}
-
-// The same collision in the scaled variable h_i = f~_i / w_i (16-bit storage):
-// moments weight h by w, the equilibrium h~eq_i = drho + rho (3 c.u + 4.5 (c.u)^2
-// - 1.5 u.u) carries no w.
-__device__ __forceinline__ float4 collide_scaled(float g[19], float omega) {
-    const float sa = HG_ADD(HG_ADD(HG_ADD(g[1], g[2]), HG_ADD(g[3], g[4])), HG_ADD(g[5], g[6]));
-    const float sd = HG_ADD(HG_ADD(HG_ADD(HG_ADD(g[7], g[8]), HG_ADD(g[9], g[10])),
-                                   HG_ADD(HG_ADD(g[11], g[12]), HG_ADD(g[13], g[14]))),
-                            HG_ADD(HG_ADD(g[15], g[16]), HG_ADD(g[17], g[18])));
-    const float drho = HG_ADD(mulw<0>(g[0]), HG_ADD(mulw<1>(sa), mulw<7>(sd)));
-    const float d12 = HG_SUB(g[1], g[2]), d34 = HG_SUB(g[3], g[4]), d56 = HG_SUB(g[5], g[6]);
-    const float d78 = HG_SUB(g[7], g[8]), d910 = HG_SUB(g[9], g[10]), d1112 = HG_SUB(g[11], g[12]);
-    const float d1314 = HG_SUB(g[13], g[14]), d1516 = HG_SUB(g[15], g[16]), d1718 = HG_SUB(g[17], g[18]);
-    const float ex = HG_ADD(HG_ADD(d78, d910), HG_ADD(d1112, d1314));
-    const float ey = HG_ADD(HG_SUB(d78, d910), HG_ADD(d1516, d1718));
-    const float ez = HG_ADD(HG_SUB(d1112, d1314), HG_SUB(d1516, d1718));
-    const float jx = HG_ADD(mulw<1>(d12), mulw<7>(ex));
-    const float jy = HG_ADD(mulw<1>(d34), mulw<7>(ey));
-    const float jz = HG_ADD(mulw<1>(d56), mulw<7>(ez));
-    const Moments m = finish_moments(drho, jx, jy, jz);
-    g[0] = HG_FMA(omega, HG_SUB(m.base, g[0]), g[0]);
-    relax_pairs<true>(g, omega, m.base, m.rho, m.ux, m.uy, m.uz);
-    return make_float4(m.drho, m.ux, m.uy, m.uz);
+    pair(IC<7>{}, 8, vadd(ux, uy));
+    pair(IC<9>{}, 10, vsub(ux, uy));
+    pair(IC<11>{}, 12, vadd(ux, uz));
+    pair(IC<13>{}, 14, vsub(ux, uz));
+    pair(IC<15>{}, 16, vadd(uy, uz));
+    pair(IC<17>{}, 18, vsub(uy, uz));
+    return {drho, ux, uy, uz};
 }
 
 template <int S> __device__ __forceinline__ float4 collide_s(float g[19], float omega) {
-    if constexpr (St<S>::kScaled) return collide_scaled(g, omega);
-    else return collide(g, omega);
+    const MomT<float> m = collide_v<St<S>::kScaled>(g, omega, 0);
+    return make_float4(m.drho, m.ux, m.uy, m.uz);
+}
+__device__ __forceinline__ float4 mom_lo(const MomT<F2> &m) {
+    return make_float4(lo2(m.drho), lo2(m.ux), lo2(m.uy), lo2(m.uz));
+}
+__device__ __forceinline__ float4 mom_hi(const MomT<F2> &m) {
+    return make_float4(hi2(m.drho), hi2(m.ux), hi2(m.uy), hi2(m.uz));
 }
 
-
-// A pointer the compiler cannot see through: loads from it are not merged with
-// earlier loads from the same address.
-template <typename T> __device__ __forceinline__ const T *opaque_ptr(const T *p) {
-    const T *q;
-    asm volatile("mov.b64 %0, %1;" : "=l"(q) : "l"(p));
-    return q;
-}
 
 template <typename T> __device__ __forceinline__ T ldg_nc(const T *p) { return __ldg(p); }
 template <> __device__ __forceinline__ __half ldg_nc(const __half *p) {
@@ -269,15 +310,9 @@ template <bool HINT, typename T> __device__ __forceinline__ T load_rw(const T *p
 }
 
 // ---- neighbour entries of a site: the 18-row table or its run encoding ----
-// Both give the same int32 entry for link I (1..18): the fluid neighbour's device
-// index, or for a non-fluid link the virtual index s + dd np with dd = opp(I) - I
-// (A/B) or I - opp(I) (AA).  TabNb reads row I-1 of the table (72 bytes per site
-// in all); RunNb reads one word per site (non-fluid flags, run within the chunk),
-// the chunk's first run and the run's 80-byte row of offsets, which the run's other
-// sites also read (L1 hits): about 4 + 80 / run-length bytes per site.
-// RunNb::reload() gives an accessor whose next reads are not merged with earlier
-// ones, so a scatter after the collision re-reads (cache hits) instead of keeping
-// 18 entries in registers.
+// The table (72 bytes per site) gives for link I (1..18) the fluid neighbour's device
+// index, or for a non-fluid link the virtual index s + dd np with dd = opp(I) - I (A/B)
+// or I - opp(I) (AA).
 template <bool HINT> struct TabNb {
     const int32_t *p;
     int64_t np;
@@ -287,75 +322,39 @@ template <bool HINT> struct TabNb {
         for (int i = 0; i < 18; ++i) nb[i] = load_nbr<HINT>(p + (int64_t)i * np);
     }
 };
-template <int SCHEME, bool HINT> struct RunNb {
-    uint32_t w;
-    const int32_t *rd;
-    int32_t s, np;
-    __device__ __forceinline__ RunNb(const DomDev &D, int64_t s_) : s((int32_t)s_), np((int32_t)D.np) {
-        w = (uint32_t)load_nbr<HINT>(reinterpret_cast<const int32_t *>(D.lword) + s_);
-        rd = D.rdelta + (int64_t)(__ldg(D.run0 + (s_ >> 10)) + (int32_t)(w >> 18)) * kRunStride;
-    }
-    __device__ __forceinline__ RunNb(uint32_t w_, const int32_t *rd_, int32_t s_, int32_t np_)
-        : w(w_), rd(rd_), s(s_), np(np_) {}
-    // all 18 entries: the run's row as five 16-byte loads
-    __device__ __forceinline__ void all(int32_t nb[18]) const {
-        int32_t d[kRunStride];
-#pragma unroll
-        for (int k = 0; k < kRunStride / 4; ++k) {
-            const int4 v = __ldg(reinterpret_cast<const int4 *>(rd) + k);
-            d[4 * k] = v.x;
-            d[4 * k + 1] = v.y;
-            d[4 * k + 2] = v.z;
-            d[4 * k + 3] = v.w;
-        }
-        unroll<1, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            constexpr int dd = SCHEME == kAA ? I - OPP(I) : OPP(I) - I;
-            nb[I - 1] = ((w >> (I - 1)) & 1u) ? s + dd * np : s + d[I - 1];
-        });
-    }
-    __device__ __forceinline__ RunNb reload() const { return RunNb(w, opaque_ptr(rd), s, np); }
-    // bring the run's row into L1 ahead of all(): its 80 bytes span at most two lines
-    __device__ __forceinline__ void prefetch() const {
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(rd));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(rd + kRunStride - 1));
-    }
-};
-// The same for a pair of adjacent sites s, s+1 (s even: both in one 1024-site
-// chunk): one 8-byte load of both table entries, or of both words; a run shared
-// by the two (the usual case) is read once.
-template <bool HINT> struct TabNb2 {
-    const int32_t *p;
-    int64_t np;
-    __device__ __forceinline__ TabNb2(const DomDev &D, int64_t s) : p(D.nbr + s), np(D.np) {}
-    template <int I> __device__ __forceinline__ int2 at() const {
-        return __ldg(reinterpret_cast<const int2 *>(p + (int64_t)(I - 1) * np));
-    }
-};
-template <int SCHEME> struct RunNb2 {
-    uint32_t wa, wb;
-    const int32_t *ra, *rb;
-    int32_t s, np;
-    __device__ __forceinline__ RunNb2(const DomDev &D, int64_t s_) : s((int32_t)s_), np((int32_t)D.np) {
-        const uint2 w = __ldg(reinterpret_cast<const uint2 *>(D.lword + s_));
-        const int32_t r0 = __ldg(D.run0 + (s_ >> 10));
-        wa = w.x;
-        wb = w.y;
-        ra = D.rdelta + (int64_t)(r0 + (int32_t)(w.x >> 18)) * kRunStride;
-        rb = D.rdelta + (int64_t)(r0 + (int32_t)(w.y >> 18)) * kRunStride;
-    }
-    template <int I> __device__ __forceinline__ int2 at() const {
-        constexpr int dd = SCHEME == kAA ? I - OPP(I) : OPP(I) - I;
-        const int32_t da = __ldg(ra + (I - 1));
-        const int32_t db = ra == rb ? da : __ldg(rb + (I - 1));
-        return make_int2(((wa >> (I - 1)) & 1u) ? s + dd * np : s + da,
-                         ((wb >> (I - 1)) & 1u) ? s + 1 + dd * np : s + 1 + db);
-    }
-};
-template <int SCHEME, bool HINT, bool RUNS>
-using NbOf = typename std::conditional<RUNS, RunNb<SCHEME, HINT>, TabNb<HINT>>::type;
-template <int SCHEME, bool RUNS>
-using Nb2Of = typename std::conditional<RUNS, RunNb2<SCHEME>, TabNb2<false>>::type;
+// The run encoding: a word per site (non-fluid flags, run within the chunk), the
+// chunk's first run, and the run's 80-byte row, which the run's other sites also read
+// (L1 hits): about 4 + 80 / run-length bytes per site.  Rows 2k+1 and 2k+2 of the
+// distributions are the two directions of one opposite pair, so both places a link can
+// read or write -- the neighbour's row and the own site's opposite row -- lie in one
+// pair: the run's row holds for every link the element offset of the fluid place from the
+// own site in the pair's first row, and a flagged link takes 0 or np instead: a select, one
+// 32 x 32 + 64-bit multiply-add and the load.
+// Link I's element offset from the own site in the first row of its pair (d = the run row's
+// entry, w = the site's word).  Flagged: the own site in the opposite row (A/B) or the own row
+// (AA, whose odd step gathers row OPP(I)).
+template <int SCHEME, int I> __device__ __forceinline__ int32_t run_offset(uint32_t w, int32_t d, int32_t np) {
+    constexpr bool second = SCHEME == kAB ? (I & 1) != 0 : (I & 1) == 0;
+    return ((w >> (I - 1)) & 1u) ? (second ? np : 0) : d;
+}
+// f(IC<I>, entry) for links I = 4 K + 1 .. 4 K + 4 (up to 18) from the run row's K-th 16 bytes.
+template <int K, typename F> __device__ __forceinline__ void run_links4(const int32_t *row, F &&f) {
+    const int4 v = __ldg(reinterpret_cast<const int4 *>(row) + K);
+    const int32_t d[4] = {v.x, v.y, v.z, v.w};
+    unroll<0, (K < 4 ? 4 : 2)>([&](auto jc) {
+        constexpr int J = decltype(jc)::v;
+        f(IC<4 * K + J + 1>{}, d[J]);
+    });
+}
+// Row I of the distributions at p (np values, npb bytes, per row): one multiply-add.
+template <int I, typename T> __device__ __forceinline__ T *row_at(T *p, uint32_t npb) {
+    using C = typename std::conditional<std::is_const<T>::value, const char, char>::type;
+    return (T *)((C *)p + (uint64_t)npb * (uint32_t)I);
+}
+// The first row of link I's opposite pair.
+template <int I, typename T> __device__ __forceinline__ T *pair_row(T *p, uint32_t npb) {
+    return row_at<(I - 1) / 2 * 2 + 1>(p, npb);
+}
 
 // ---- sites next to an iolet (rare path) ----
 // Neighbour table entries of non-fluid links hold a virtual index that makes
@@ -371,12 +370,12 @@ __device__ __forceinline__ int site_slot(const DomDev &D, int64_t s, uint32_t wo
     return __ldg(D.ioprefix + (s >> 5)) + __popc(word & ((1u << (s & 31)) - 1u));
 }
 template <int S>
-__device__ __forceinline__ void apply_iolet_links(const DomDev &D, int slot, float g[19]) {
+__device__ __forceinline__ void apply_iolet_links(const DomDev &D, const float *bcv, int slot, float g[19]) {
     const int32_t *codes = D.io_codes + (int64_t)slot * 18;
     unroll<1, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
         const int32_t c = __ldg(codes + (I - 1));
-        if (c < -1) g[I] = iolet_rule<I, St<S>::kScaled>(D, -c - 2, slot, g[I]);
+        if (c < -1) g[I] = iolet_rule<I, St<S>::kScaled>(D, bcv, -c - 2, slot, g[I]);
     });
 }
 // A stream-collide launch may start while the previous step's iolet update is
@@ -395,8 +394,39 @@ __device__ __forceinline__ int iolet_fixup(const DomDev &D, int64_t s, float g[1
     if (!site_flag(D, s, word)) return -1;
     wait_for_iolet_update();
     const int slot = site_slot(D, s, word);
-    apply_iolet_links<S>(D, slot, g);
+    apply_iolet_links<S>(D, D.bcv, slot, g);
     return slot;
+}
+// The same for one half of a packed pair (HI: the second site); the caller found the flag.
+template <int S, bool HI>
+__device__ __forceinline__ void iolet_links_half(const DomDev &D, const float *bcv, int slot, F2 g[19]) {
+    const int32_t *codes = D.io_codes + (int64_t)slot * 18;
+    unroll<1, 19>([&](auto ic) {
+        constexpr int I = decltype(ic)::v;
+        const int32_t c = __ldg(codes + (I - 1));
+        if (c < -1) {
+            const float v = iolet_rule<I, St<S>::kScaled>(D, bcv, -c - 2, slot, HI ? hi2(g[I]) : lo2(g[I]));
+            g[I] = HI ? pk2(lo2(g[I]), v) : pk2(v, hi2(g[I]));
+        }
+    });
+}
+template <int S>
+__device__ __forceinline__ void iolet_fixup2(const DomDev &D, int64_t sa, int64_t sb, F2 g[19], int &slot_a,
+                                             int &slot_b) {
+    uint32_t wa, wb;
+    const bool fa = site_flag(D, sa, wa), fb = site_flag(D, sb, wb);
+    slot_a = slot_b = -1;
+    if (fa || fb) {
+        wait_for_iolet_update();
+        if (fa) {
+            slot_a = site_slot(D, sa, wa);
+            iolet_links_half<S, false>(D, D.bcv, slot_a, g);
+        }
+        if (fb) {
+            slot_b = site_slot(D, sb, wb);
+            iolet_links_half<S, true>(D, D.bcv, slot_b, g);
+        }
+    }
 }
 
 template <typename T> __device__ __forceinline__ T *opaque(T *p) {
@@ -405,19 +435,14 @@ template <typename T> __device__ __forceinline__ T *opaque(T *p) {
     return q;
 }
 
-// ---- A/B pull: F_{t-1} in src, F_t to dst ----
-template <int S, bool HINT = false, bool RUNS = false>
+// ---- A/B pull: F_{t-1} in src, F_t to dst (18-row table) ----
+template <int S, bool HINT = false>
 __device__ __forceinline__ void site_ab(const DomDev &D, const typename St<S>::T *__restrict__ src,
-                                        typename St<S>::T *__restrict__ dst, int64_t s);
-
-// The A/B site update with the site's neighbour accessor already made.
-template <int S, bool HINT, typename NB>
-__device__ __forceinline__ void site_ab_with(const DomDev &D, const typename St<S>::T *__restrict__ src,
-                                             typename St<S>::T *__restrict__ dst, int64_t s, const NB &tab) {
+                                        typename St<S>::T *__restrict__ dst, int64_t s) {
     using Tr = St<S>;
     const int64_t np = D.np;
     int32_t nb[18];
-    tab.all(nb);
+    TabNb<HINT>(D, s).all(nb);
     float g[19];
     g[0] = Tr::template ld<0>(load_ro<HINT>(src + s));
     unroll<1, 19>([&](auto ic) {  // virtual indices: walls read their own opposite value
@@ -431,12 +456,6 @@ __device__ __forceinline__ void site_ab_with(const DomDev &D, const typename St<
         dst[(int64_t)I * np + s] = Tr::template st<I>(g[I]);
     });
     if (slot >= 0) D.bnd[slot] = m;
-}
-
-template <int S, bool HINT, bool RUNS>
-__device__ __forceinline__ void site_ab(const DomDev &D, const typename St<S>::T *__restrict__ src,
-                                        typename St<S>::T *__restrict__ dst, int64_t s) {
-    site_ab_with<S, HINT>(D, src, dst, s, NbOf<kAB, HINT, RUNS>(D, s));
 }
 
 // ---- AA even step: state G_t natural at the own site -> F_t swapped at the own site ----
@@ -465,19 +484,12 @@ __device__ __forceinline__ void site_aa_even(const DomDev &D, typename St<S>::T 
 // ---- AA odd step: gather F_{t-1} (swapped) from x - c_i, scatter F_t to x + c_i ----
 // Entry OPP(I) of the site's row is the site at x + c_I; its virtual index for
 // a non-fluid link turns the scatter into the raw write to the own slot OPP(I).
-template <int S, bool HINT, bool RUNS, bool STASH, typename NB>
-__device__ __forceinline__ void site_aa_odd_with(const DomDev &D, typename St<S>::T *buf, int64_t s,
-                                                 const NB &tab, int32_t *stash = nullptr) {
+template <int S, bool HINT = false>
+__device__ __forceinline__ void site_aa_odd(const DomDev &D, typename St<S>::T *buf, int64_t s) {
     using Tr = St<S>;
     const int64_t np = D.np;
     int32_t nb[18];
-    tab.all(nb);
-    if constexpr (STASH) {  // 19 words per thread (odd stride: no bank conflicts), 18 used
-        stash += 19 * threadIdx.x;
-#pragma unroll
-        for (int i = 0; i < 18; ++i) stash[i] = nb[i];
-        asm volatile("" ::: "memory");  // the stash stores stay ahead of the gathers
-    }
+    TabNb<HINT>(D, s).all(nb);
     float g[19];
     g[0] = Tr::template ld<0>(load_rw<HINT>(buf + s));
     unroll<1, 19>([&](auto ic) {
@@ -487,40 +499,13 @@ __device__ __forceinline__ void site_aa_odd_with(const DomDev &D, typename St<S>
     const int slot = iolet_fixup<S>(D, s, g);
     const float4 m = collide_s<S>(g, D.omega);
     typename St<S>::T *wb = opaque(buf);
-    // the scatter addresses are the gather addresses (entry OPP(I) of the site at x +
-    // c_I): STASH takes the 18 entries back from shared memory, otherwise they are
-    // decoded again (cache hits); either frees 18 registers across the collision
     wb[s] = Tr::template st<0>(g[0]);
-    if constexpr (RUNS || STASH) {
-        if constexpr (STASH) {
-            // the stash address is known only once the collision has produced m: the
-            // reads cannot move above it, so the entries are not live across it
-            int32_t *st2;
-            asm volatile("{\n\t.reg .f32 t;\n\tmov.f32 t, %2;\n\tmov.b64 %0, %1;\n\t}"
-                         : "=l"(st2) : "l"(stash), "f"(m.x) : "memory");
-#pragma unroll
-            for (int i = 0; i < 18; ++i) nb[i] = st2[i];
-        } else {
-            tab.reload().all(nb);
-        }
-        unroll<1, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            wb[(int64_t)I * np + nb[OPP(I) - 1]] = Tr::template st<I>(g[I]);
-        });
-    } else {  // table: each store's entry reread right before it
-        const int32_t *nb2 = opaque(D.nbr);
-        unroll<1, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            wb[(int64_t)I * np + __ldg(nb2 + (int64_t)(OPP(I) - 1) * np + s)] = Tr::template st<I>(g[I]);
-        });
-    }
+    const int32_t *nb2 = opaque(D.nbr);  // each store's entry reread right before it (cache hit)
+    unroll<1, 19>([&](auto ic) {
+        constexpr int I = decltype(ic)::v;
+        wb[(int64_t)I * np + __ldg(nb2 + (int64_t)(OPP(I) - 1) * np + s)] = Tr::template st<I>(g[I]);
+    });
     if (slot >= 0) D.bnd[slot] = m;
-}
-
-template <int S, bool HINT = false, bool RUNS = false, bool STASH = false>
-__device__ __forceinline__ void site_aa_odd(const DomDev &D, typename St<S>::T *buf, int64_t s,
-                                            int32_t *stash = nullptr) {
-    site_aa_odd_with<S, HINT, RUNS, STASH>(D, buf, s, NbOf<kAA, HINT, RUNS>(D, s), stash);
 }
 
 // ==== async-staged variant (V = 1) ==========================================
@@ -766,35 +751,45 @@ template <> struct Pair16<kBF16> {
 template <> struct Pair<kF16> : Pair16<kF16> {};
 template <> struct Pair<kBF16> : Pair16<kBF16> {};
 
+template <int S, int I> __device__ __forceinline__ F2 ld_pair(const typename St<S>::T *p) {
+    float a, b;
+    Pair<S>::template ld<I>(p, a, b);
+    return pk2(a, b);
+}
+template <int S, int I> __device__ __forceinline__ void st_pair(typename St<S>::T *p, F2 v) {
+    Pair<S>::template st<I>(p, lo2(v), hi2(v));
+}
+__device__ __forceinline__ void put_moments(const DomDev &D, int slot_a, int slot_b, const MomT<F2> &m) {
+    if (slot_a >= 0) D.bnd[slot_a] = mom_lo(m);
+    if (slot_b >= 0) D.bnd[slot_b] = mom_hi(m);
+}
+
 // ---- A/B pull on a pair of adjacent sites (variant 5, 16-bit storage) ----
 // Sites s and s+1 (s even) share one 8-byte load per neighbour-table row, one
 // 4-byte load of the rest values and one 4-byte store per direction: fewer
 // memory instructions per site for a kernel that runs near its issue limit.
-template <int S, bool RUNS = false>
+template <int S>
 __device__ __forceinline__ void site_ab_pair(const DomDev &D, const typename St<S>::T *__restrict__ src,
                                              typename St<S>::T *__restrict__ dst, int64_t s) {
     using Tr = St<S>;
     const int64_t np = D.np;
-    const Nb2Of<kAB, RUNS> tab(D, s);
-    float ga[19], gb[19];
-    Pair<S>::template ld<0>(src + s, ga[0], gb[0]);
+    F2 g[19];
+    g[0] = ld_pair<S, 0>(src + s);
     unroll<1, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
-        const int2 nb = tab.template at<I>();
-        ga[I] = Tr::template ld<I>(ldg_nc(src + ((int64_t)I * np + nb.x)));
-        gb[I] = Tr::template ld<I>(ldg_nc(src + ((int64_t)I * np + nb.y)));
+        const int2 nb = __ldg(reinterpret_cast<const int2 *>(D.nbr + (int64_t)(I - 1) * np + s));
+        g[I] = pk2(Tr::template ld<I>(ldg_nc(src + ((int64_t)I * np + nb.x))),
+                   Tr::template ld<I>(ldg_nc(src + ((int64_t)I * np + nb.y))));
     });
-    const int slot_a = iolet_fixup<S>(D, s, ga);
-    const int slot_b = iolet_fixup<S>(D, s + 1, gb);
-    const float4 ma = collide_s<S>(ga, D.omega);
-    const float4 mb = collide_s<S>(gb, D.omega);
+    int slot_a, slot_b;
+    iolet_fixup2<S>(D, s, s + 1, g, slot_a, slot_b);
+    const MomT<F2> m = collide_v<Tr::kScaled>(g, D.omega, D.neg_zero2);
     typename St<S>::T *wb = opaque(dst + s);
     unroll<0, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
-        Pair<S>::template st<I>(wb + (int64_t)I * np, ga[I], gb[I]);
+        st_pair<S, I>(wb + (int64_t)I * np, g[I]);
     });
-    if (slot_a >= 0) D.bnd[slot_a] = ma;
-    if (slot_b >= 0) D.bnd[slot_b] = mb;
+    put_moments(D, slot_a, slot_b, m);
 }
 
 // ---- AA on a pair of adjacent sites (variant 6 / 7: 7 adds L2 prefetch hints) ----
@@ -806,80 +801,151 @@ template <int S, bool HINT>
 __device__ __forceinline__ void site_aa_odd_pair(const DomDev &D, typename St<S>::T *buf, int64_t s) {
     using Tr = St<S>;
     const int64_t np = D.np;
-    float ga[19], gb[19];
-    Pair<S>::template ld<0>(buf + s, ga[0], gb[0]);
+    F2 g[19];
+    g[0] = ld_pair<S, 0>(buf + s);
     unroll<1, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
         const int2 nb = __ldg(reinterpret_cast<const int2 *>(D.nbr + (int64_t)(I - 1) * np + s));
-        ga[I] = Tr::template ld<I>(load_rw<HINT>(buf + ((int64_t)OPP(I) * np + nb.x)));
-        gb[I] = Tr::template ld<I>(load_rw<HINT>(buf + ((int64_t)OPP(I) * np + nb.y)));
+        g[I] = pk2(Tr::template ld<I>(load_rw<HINT>(buf + ((int64_t)OPP(I) * np + nb.x))),
+                   Tr::template ld<I>(load_rw<HINT>(buf + ((int64_t)OPP(I) * np + nb.y))));
     });
-    const int slot_a = iolet_fixup<S>(D, s, ga);
-    const int slot_b = iolet_fixup<S>(D, s + 1, gb);
-    const float4 ma = collide_s<S>(ga, D.omega);
-    const float4 mb = collide_s<S>(gb, D.omega);
+    int slot_a, slot_b;
+    iolet_fixup2<S>(D, s, s + 1, g, slot_a, slot_b);
+    const MomT<F2> m = collide_v<Tr::kScaled>(g, D.omega, D.neg_zero2);
     typename St<S>::T *wb = opaque(buf);
     const int32_t *nb2 = opaque(D.nbr);  // reread (L1 hits) instead of keeping 36 entries live
-    Pair<S>::template st<0>(wb + s, ga[0], gb[0]);
+    st_pair<S, 0>(wb + s, g[0]);
     unroll<1, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
         const int2 tg = __ldg(reinterpret_cast<const int2 *>(nb2 + (int64_t)(OPP(I) - 1) * np + s));
-        wb[(int64_t)I * np + tg.x] = Tr::template st<I>(ga[I]);
-        wb[(int64_t)I * np + tg.y] = Tr::template st<I>(gb[I]);
+        wb[(int64_t)I * np + tg.x] = Tr::template st<I>(lo2(g[I]));
+        wb[(int64_t)I * np + tg.y] = Tr::template st<I>(hi2(g[I]));
     });
-    if (slot_a >= 0) D.bnd[slot_a] = ma;
-    if (slot_b >= 0) D.bnd[slot_b] = mb;
+    put_moments(D, slot_a, slot_b, m);
 }
 
-// AA even step on the same pairs: local, vector loads and stores of both sites.
-template <int S, bool HINT>
+// AA even step on adjacent pairs: local, vector loads and stores of both sites.
+template <int S>
 __device__ __forceinline__ void site_aa_even_pair(const DomDev &D, typename St<S>::T *buf, int64_t s) {
     const int64_t np = D.np;
-    float ga[19], gb[19];
+    F2 g[19];
     unroll<0, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
-        Pair<S>::template ld<I>(buf + (int64_t)I * np + s, ga[I], gb[I]);
+        g[I] = ld_pair<S, I>(buf + (int64_t)I * np + s);
     });
-    const int slot_a = iolet_fixup<S>(D, s, ga);
-    const int slot_b = iolet_fixup<S>(D, s + 1, gb);
-    const float4 ma = collide_s<S>(ga, D.omega);
-    const float4 mb = collide_s<S>(gb, D.omega);
+    int slot_a, slot_b;
+    iolet_fixup2<S>(D, s, s + 1, g, slot_a, slot_b);
+    const MomT<F2> m = collide_v<St<S>::kScaled>(g, D.omega, D.neg_zero2);
     typename St<S>::T *wb = opaque(buf + s);
     unroll<0, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
-        Pair<S>::template st<I>(wb + (int64_t)OPP(I) * np, ga[I], gb[I]);
+        st_pair<S, I>(wb + (int64_t)OPP(I) * np, g[I]);
     });
-    if (slot_a >= 0) D.bnd[slot_a] = ma;
-    if (slot_b >= 0) D.bnd[slot_b] = mb;
+    put_moments(D, slot_a, slot_b, m);
 }
 
 template <int S>
 __device__ __forceinline__ void tile_aa_even_pairs(const DomDev &D, const TileDev &tl) {
     using T = typename St<S>::T;
     T *buf = (T *)D.f[0];
-    const int64_t np = D.np;
     for (int r = 2 * threadIdx.x; r < tl.count; r += 2 * blockDim.x) {
-        const int64_t s = tl.start + r;  // even: tiles start at multiples of 64
-        if (r + 1 >= tl.count) {         // ragged tail: one site
-            site_aa_even<S>(D, buf, s);
-            continue;
+        const int64_t s = tl.start + r;  // even: tiles start at multiples of 32
+        if (r + 1 >= tl.count) site_aa_even<S>(D, buf, s);  // ragged tail: one site
+        else site_aa_even_pair<S>(D, buf, s);
+    }
+}
+
+// ==== run-encoded form (variants 8..14) ========================================
+// What bounds it: for 16-bit storage instruction issue (68 % of the slots; 438 instructions
+// per site and A/B step, 518 before the links were decoded as below), for FP32 HBM (A/B) and
+// the misaligned scatter (AA odd).  40 registers, so 48 warps per SM hide the chain word ->
+// run row -> gathers.  ~10M-site tree, stream-collide alone, before -> now: FP32 A/B 243 ->
+// 241 us, FP16 A/B 192 -> 181, FP32 AA odd 303 -> 272, FP16 AA odd 236 -> 198 (even 123).
+// Tried and slower: two sites per thread with packed arithmetic (350 instructions per site,
+// but 64-90 registers: 188-230 us FP16 A/B); lists of all-fluid pairs and single sites (250
+// instructions per site, but the lists' stores leave sectors half written: FP32 A/B 296 us);
+// an L2 prefetch of the rows 64K..1M sites ahead (no change to 20 % slower).
+template <int S, int SCHEME> __device__ __forceinline__ float run_ld(const typename St<S>::T *p) {
+    if constexpr (SCHEME == kAA) return St<S>::template ld<0>(load_rw<true>(p));
+    else return St<S>::template ld<0>(load_ro<true>(p));
+}
+struct RunSite {
+    uint32_t w;
+    const int32_t *row;
+};
+__device__ __forceinline__ RunSite run_site(const DomDev &D, int64_t s) {
+    RunSite r;
+    r.w = (uint32_t)load_nbr<true>(reinterpret_cast<const int32_t *>(D.lword) + s);
+    r.row = D.rdelta + (int64_t)(__ldg(D.run0 + (s >> 10)) + (int32_t)((r.w >> 18) & 1023u)) * kRunStride;
+    return r;
+}
+// A/B step or AA odd step of one site whose word and run row are at hand.  The AA scatter
+// goes to the places the gather read (direction I where its opposite was read); their 18
+// offsets wait in shared memory, one bank per thread, instead of being decoded again.
+template <int S, int SCHEME>
+__device__ __forceinline__ void site_run(const DomDev &D, const typename St<S>::T *src, typename St<S>::T *dst,
+                                         int64_t s, const RunSite &r, int32_t *stash) {
+    using Tr = St<S>;
+    using T = typename Tr::T;
+    const int32_t np = (int32_t)D.np;
+    const uint32_t npb = (uint32_t)D.np * sizeof(T);
+    const T *p = src + s;
+    float g[19];
+    g[0] = run_ld<S, SCHEME>(p);
+    unroll<0, 5>([&](auto kc) {
+        run_links4<decltype(kc)::v>(r.row, [&](auto ic, int32_t d) {
+            constexpr int I = decltype(ic)::v;
+            const int32_t off = run_offset<SCHEME, I>(r.w, d, np);
+            g[I] = run_ld<S, SCHEME>(pair_row<I>(p, npb) + off);
+            if constexpr (SCHEME == kAA) stash[(I - 1) * blockDim.x] = off;
+        });
+    });
+    int slot = -1;
+    if (r.w >> 31) {  // a link into an iolet opening
+        wait_for_iolet_update();
+        slot = site_slot(D, s, __ldg(D.iomask + (s >> 5)));
+        apply_iolet_links<S>(D, D.bcv, slot, g);
+    }
+    const float4 m = collide_s<S>(g, D.omega);
+    int32_t *back = stash;
+    if constexpr (SCHEME == kAA)
+        // the address is known only once the collision has produced m: the reads cannot
+        // move above it, so the 18 offsets are not live across it
+        asm volatile("{\n\t.reg .f32 t;\n\tmov.f32 t, %2;\n\tmov.b64 %0, %1;\n\t}"
+                     : "=l"(back) : "l"(stash), "f"(m.x) : "memory");
+    T *q = opaque(dst + s);
+    *q = Tr::template st<0>(g[0]);
+    unroll<1, 19>([&](auto ic) {
+        constexpr int I = decltype(ic)::v;
+        const T v = Tr::template st<I>(g[I]);
+        if constexpr (SCHEME == kAB) *row_at<I>(q, npb) = v;
+        else pair_row<I>(q, npb)[back[(OPP(I) - 1) * blockDim.x]] = v;
+    });
+    if (slot >= 0) D.bnd[slot] = m;
+}
+// A tile of SPT * blockDim sites; with SPT = 2 both words are loaded, and both run rows
+// prefetched into L1 (80 bytes: at most two lines), before the first site's gathers.
+template <int S, int SCHEME, int SPT>
+__device__ __forceinline__ void tile_runs(const DomDev &D, const TileDev &tl, const typename St<S>::T *src,
+                                          typename St<S>::T *dst, int32_t *stash) {
+    RunSite r[SPT];
+#pragma unroll
+    for (int j = 0; j < SPT; ++j) {
+        const int q = j * blockDim.x + threadIdx.x;
+        r[j].w = 0;
+        r[j].row = D.rdelta;
+        if (q < tl.count) {
+            r[j] = run_site(D, tl.start + q);
+            if constexpr (SPT > 1) {
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(r[j].row));
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(r[j].row + kRunStride - 1));
+            }
         }
-        float ga[19], gb[19];
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            Pair<S>::template ld<I>(buf + (int64_t)I * np + s, ga[I], gb[I]);
-        });
-        const int slot_a = iolet_fixup<S>(D, s, ga);
-        const int slot_b = iolet_fixup<S>(D, s + 1, gb);
-        const float4 ma = collide_s<S>(ga, D.omega);
-        const float4 mb = collide_s<S>(gb, D.omega);
-        T *wb = opaque(buf + s);
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            Pair<S>::template st<I>(wb + (int64_t)OPP(I) * np, ga[I], gb[I]);
-        });
-        if (slot_a >= 0) D.bnd[slot_a] = ma;
-        if (slot_b >= 0) D.bnd[slot_b] = mb;
+    }
+#pragma unroll
+    for (int j = 0; j < SPT; ++j) {
+        const int q = j * blockDim.x + threadIdx.x;
+        if (q < tl.count) site_run<S, SCHEME>(D, src, dst, tl.start + q, r[j], stash + threadIdx.x);
     }
 }
 
@@ -979,12 +1045,26 @@ __device__ __forceinline__ void tile_aa_even_tma(const DomDev &D, const TileDev 
 // PAR is the parity of the step this launch executes: 0 = even, 1 = odd (the
 // AA step kind), 2 = read from the domain's step counter per block (A/B, and AA
 // batches whose domains are at different parities).
-// One tile of one domain, after the prologue has located it.
-template <int S, int SCHEME, int SPT, int PAR, int V, bool RUNS, bool STASH = false, bool HOIST = false>
-__device__ __forceinline__ void stream_collide_tile_impl(const DomDev &D, const TileDev &tl, bool odd,
-                                                         uint32_t *stage) {
+// One tile of one domain, after the prologue has located it.  Variants 8..14 are one kernel
+// (V = 8), which reads the run-encoded neighbour table.  The host launches it only on domains
+// that have one (the others get a table form); a domain without one here is reported through
+// the error word (code 2) and left untouched.
+constexpr bool hinted(int v) { return v == 3 || v == 7; }
+template <int S, int SCHEME, int SPT, int PAR, int V>
+__device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileDev &tl, bool odd,
+                                                    uint32_t *stage) {
     using T = typename St<S>::T;
-    if constexpr (V == 1 || V == 2 || V == 4) {
+    constexpr bool HINT = hinted(V);
+    if constexpr (V == 8) {
+        if (D.lword == nullptr) {
+            if (threadIdx.x == 0) atomicExch(D.err, 2);
+            return;
+        }
+        if (SCHEME == kAB || PAR == 1 || (PAR == 2 && odd))
+            tile_runs<S, SCHEME, SPT>(D, tl, (const T *)D.f[SCHEME == kAA || odd ? 0 : 1],
+                                            (T *)D.f[SCHEME == kAA || !odd ? 0 : 1], (int32_t *)stage);
+        else tile_aa_even_pairs<S>(D, tl);
+    } else if constexpr (V == 1 || V == 2 || V == 4) {
         if constexpr (SCHEME == kAB) {
             tile_ab_async<S, SPT>(D, tl, odd, stage);
         } else {
@@ -1000,26 +1080,14 @@ __device__ __forceinline__ void stream_collide_tile_impl(const DomDev &D, const 
     } else if constexpr (V == 6 || V == 7) {
         // AA on adjacent pairs: each thread takes sites 2t and 2t+1 of the tile (SPT = 2)
         static_assert(SCHEME == kAA && SPT == 2, "variants 6 and 7 are the AA pair forms");
-        constexpr bool HINT = V == 7;
         T *buf = (T *)D.f[0];
-        if (RUNS && odd) {
-            // the run-encoded odd step takes one site at a time (decoding two runs at
-            // once keeps too many values live), sites t and t + blockDim, so a warp's
-            // gathers and scatters cover consecutive sites
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int r = j * blockDim.x + threadIdx.x;
-                if (r < tl.count) site_aa_odd<S, HINT, true, STASH>(D, buf, tl.start + r, (int32_t *)stage);
-            }
-            return;
-        }
         const int r = 2 * threadIdx.x;
         const int64_t s = tl.start + r;  // even: tiles start at multiples of 2 * blockDim
         if (r + 1 < tl.count) {
             if (odd) site_aa_odd_pair<S, HINT>(D, buf, s);
-            else site_aa_even_pair<S, HINT>(D, buf, s);
+            else site_aa_even_pair<S>(D, buf, s);
         } else if (r < tl.count) {  // ragged tail: one site
-            if (odd) site_aa_odd<S, HINT, false>(D, buf, s);
+            if (odd) site_aa_odd<S, HINT>(D, buf, s);
             else site_aa_even<S, HINT>(D, buf, s);
         }
     } else if constexpr (V == 5) {
@@ -1029,85 +1097,21 @@ __device__ __forceinline__ void stream_collide_tile_impl(const DomDev &D, const 
         const int64_t s = tl.start + r;  // even: tiles start at multiples of 2 * blockDim
         const T *src = (const T *)D.f[odd ? 0 : 1];
         T *dst = (T *)D.f[odd ? 1 : 0];
-        if (r + 1 < tl.count) site_ab_pair<S, RUNS>(D, src, dst, s);
-        else if (r < tl.count) site_ab<S, false, RUNS>(D, src, dst, s);  // ragged tail: one site
-    } else if (HOIST && (SCHEME == kAB || odd)) {
-        // every site's link word first (and a prefetch of its run row into L1), then the
-        // sites one by one: a later site's decode no longer waits on its own word and row
-        constexpr bool HINT = V == 3;
-        uint32_t ws[SPT];
-        const int32_t *rds[SPT];
+        if (r + 1 < tl.count) site_ab_pair<S>(D, src, dst, s);
+        else if (r < tl.count) site_ab<S>(D, src, dst, s);  // ragged tail: one site
+    } else {
 #pragma unroll
         for (int j = 0; j < SPT; ++j) {
             const int r = j * blockDim.x + threadIdx.x;
-            ws[j] = 0;
-            rds[j] = D.rdelta;
-            if (r < tl.count) {
-                const RunNb<SCHEME, HINT> t(D, tl.start + r);
-                t.prefetch();
-                ws[j] = t.w;
-                rds[j] = t.rd;
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < SPT; ++j) {
-            const int r = j * blockDim.x + threadIdx.x;
+            const int64_t s = tl.start + r;
             if (r >= tl.count) continue;
-            const int64_t s = tl.start + r;
-            const RunNb<SCHEME, HINT> t(ws[j], rds[j], (int32_t)s, (int32_t)D.np);
             if constexpr (SCHEME == kAB) {
-                site_ab_with<S, HINT>(D, (const T *)D.f[odd ? 0 : 1], (T *)D.f[odd ? 1 : 0], s, t);
+                site_ab<S, HINT>(D, (const T *)D.f[odd ? 0 : 1], (T *)D.f[odd ? 1 : 0], s);
             } else {
-                site_aa_odd_with<S, HINT, true, false>(D, (T *)D.f[0], s, t);
+                if (odd) site_aa_odd<S, HINT>(D, (T *)D.f[0], s);
+                else site_aa_even<S, HINT>(D, (T *)D.f[0], s);
             }
         }
-    } else {
-        constexpr bool HINT = V == 3;
-#pragma unroll
-        for (int j = 0; j < SPT; ++j) {
-            const int r = j * blockDim.x + threadIdx.x;
-            const int64_t s = tl.start + r;
-            const bool live = r < tl.count;
-            if constexpr (SCHEME == kAB) {
-                if (live) {
-                    const T *src = (const T *)D.f[odd ? 0 : 1];
-                    T *dst = (T *)D.f[odd ? 1 : 0];
-                    site_ab<S, HINT, RUNS>(D, src, dst, s);
-                }
-            } else {
-                T *buf = (T *)D.f[0];
-                if (live) {
-                    if (odd) site_aa_odd<S, HINT, RUNS, STASH>(D, buf, s, (int32_t *)stage);
-                    else site_aa_even<S, HINT>(D, buf, s);
-                }
-            }
-        }
-    }
-}
-
-// Variants 8..11 are 3, 5, 6, 7 reading the run-encoded neighbour table.  The host
-// launches them only on domains that have one (the others get 3, 5, 6, 7); a domain
-// without one here is reported through the error word (code 2) and left untouched.
-// Variant 12 is 8 for the AA scheme with the odd step's 18 entries stashed in shared
-// memory across the collision instead of decoded twice; 14 is 10 with the same stash;
-// 13 is 8 with every site's link word loaded (and its run row prefetched) before the
-// first site's gathers.
-template <int V> constexpr int table_variant() {
-    return V == 8 || V == 12 || V == 13 ? 3 : V == 9 ? 5 : V == 10 || V == 14 ? 6 : V == 11 ? 7 : V;
-}
-
-template <int S, int SCHEME, int SPT, int PAR, int V>
-__device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileDev &tl, bool odd,
-                                                    uint32_t *stage) {
-    if constexpr (V >= 8) {
-        if (D.lword == nullptr) {
-            if (threadIdx.x == 0) atomicExch(D.err, 2);
-            return;
-        }
-        stream_collide_tile_impl<S, SCHEME, SPT, PAR, table_variant<V>(), true, V == 12 || V == 14, V == 13>(D, tl, odd,
-                                                                                                 stage);
-    } else {
-        stream_collide_tile_impl<S, SCHEME, SPT, PAR, V, false>(D, tl, odd, stage);
     }
 }
 
@@ -1137,8 +1141,8 @@ __global__ void __launch_bounds__(512) k_stream_collide(const DomDev *__restrict
 }
 
 // One domain per launch: the descriptor is a kernel parameter (constant bank)
-// and block b takes sites [b*T, b*T + T) with T = SPT * blockDim, so no block
-// waits on a table load or a barrier before its first neighbour-table load.
+// and block b takes units [b*T, b*T + T) of the n (sites, or tasks: tile_units), so no
+// block waits on a table load or a barrier before its first neighbour-table load.
 template <int S, int SCHEME, int SPT, int PAR, int V>
 __global__ void __launch_bounds__(512) k_stream_collide_one(const __grid_constant__ DomDev D, int64_t n,
                                                             int off) {
@@ -1165,8 +1169,8 @@ cudaError_t launch_sc_one(const CollideCfg &cfg, const DomDev *doms, const TileD
     // V1/V4: cp.async stage of 4-byte words (V4 reuses it for the odd step's outputs);
     // V2 also holds the even step's 19 rows + mbarrier
     size_t smem = (V == 1 || V == 2 || V == 4) ? (size_t)SPT * 19 * cfg.block * 4 : 0;
-    if (V == 12 || V == 14) smem = (size_t)19 * cfg.block * 4;  // the AA odd step's entry stash
     if (V == 2) smem += 16;
+    if (V == 8 && SCHEME == kAA && PAR != 0) smem = (size_t)18 * 4 * cfg.block;  // odd step's offsets
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)n_tiles);
     lc.blockDim = dim3((unsigned)cfg.block);
@@ -1227,45 +1231,8 @@ cudaError_t launch_sc_spt(const CollideCfg &cfg, const DomDev *doms, const TileD
         else if (cfg.variant == 6) return launch_sc_one<S, SCHEME, PAR, 6, 2>(cfg, doms, tiles, n_tiles, off, one, st);
         else return launch_sc_one<S, SCHEME, PAR, 7, 2>(cfg, doms, tiles, n_tiles, off, one, st);
     }
-    if (cfg.variant == 8) {
-        switch (cfg.spt) {
-            case 1: return launch_sc_one<S, SCHEME, PAR, 8, 1>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 2: return launch_sc_one<S, SCHEME, PAR, 8, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 4: return launch_sc_one<S, SCHEME, PAR, 8, 4>(cfg, doms, tiles, n_tiles, off, one, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (cfg.variant == 14) {
-        if constexpr (SCHEME != kAA) return cudaErrorInvalidValue;
-        else if (cfg.spt != 2) return cudaErrorInvalidValue;
-        else return launch_sc_one<S, SCHEME, PAR, 14, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-    }
-    if (cfg.variant == 13) {
-        switch (cfg.spt) {
-            case 2: return launch_sc_one<S, SCHEME, PAR, 13, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 4: return launch_sc_one<S, SCHEME, PAR, 13, 4>(cfg, doms, tiles, n_tiles, off, one, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (cfg.variant == 12) {
-        if constexpr (SCHEME != kAA) return cudaErrorInvalidValue;
-        else switch (cfg.spt) {
-            case 1: return launch_sc_one<S, SCHEME, PAR, 12, 1>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 2: return launch_sc_one<S, SCHEME, PAR, 12, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (cfg.variant == 9) {
-        if constexpr (SCHEME != kAB || S == kF32) return cudaErrorInvalidValue;
-        else if (cfg.spt != 2) return cudaErrorInvalidValue;
-        else return launch_sc_one<S, SCHEME, PAR, 9, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-    }
-    if (cfg.variant == 10 || cfg.variant == 11) {
-        if constexpr (SCHEME != kAA) return cudaErrorInvalidValue;
-        else if (cfg.spt != 2) return cudaErrorInvalidValue;
-        else if (cfg.variant == 10) return launch_sc_one<S, SCHEME, PAR, 10, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-        else return launch_sc_one<S, SCHEME, PAR, 11, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-    }
+    if (cfg.variant >= 8)
+        return launch_sc_one<S, SCHEME, PAR, 8, run_spt(S, SCHEME, PAR)>(cfg, doms, tiles, n_tiles, off, one, st);
     if (cfg.variant == 2) {
         if (SCHEME == kAB) return cudaErrorInvalidValue;
         switch (cfg.spt) {

@@ -655,6 +655,7 @@ DomDev make_domdev(hg_ctx *ctx, hg_domain *d) {
     D.err = (int32_t *)ctx->errw.p;
     D.n = d->n;
     D.np = d->np;
+    D.neg_zero2 = 0x8000000080000000ull;
     D.omega = (float)(1.0 / d->tau);
     D.n_io = d->nio;
     return D;
@@ -797,6 +798,23 @@ bool build_runs(const int32_t *nbr, int64_t n, int64_t n_ref, int64_t np, int vd
         }
     }, 1);
     return true;
+}
+
+// Run rows as the kernels read them: offsets from the own site in the first row of the
+// link's opposite pair.  A/B gathers link i from row i, AA from row opp(i): the second row
+// of the pair for even i (A/B) or odd i (AA).  Bit 31 of a word: the site has a link into
+// an iolet opening (its bit of `mask`).
+void runs_for_device(std::vector<int32_t> &rdelta, U32Table &lword, const uint32_t *mask, int64_t n, int scheme,
+                     int64_t np) {
+    parallel_for((int64_t)rdelta.size() / kRunStride, [&](int64_t lo, int64_t hi) {
+        for (int64_t r = lo; r < hi; ++r)
+            for (int i = 1; i < 19; ++i)
+                if (scheme == HG_SCHEME_AA ? (i & 1) != 0 : (i & 1) == 0)
+                    rdelta[(size_t)r * kRunStride + i - 1] += (int32_t)np;
+    });
+    parallel_for(n, [&](int64_t lo, int64_t hi) {
+        for (int64_t q = lo; q < hi; ++q) lword[(size_t)q] |= ((mask[q >> 5] >> (q & 31)) & 1u) << 31;
+    });
 }
 
 // Canonical site order (ascending 3-D Morton key) and neighbour table in
@@ -1162,8 +1180,10 @@ int hg_domain_create(hg_ctx *ctx, const int32_t *xyz, int64_t n, const hg_iolet 
     trace.mark("virtual indices");
     U32Table lword;
     std::vector<int32_t> run0, rdelta;
-    if (build_runs(nbr.data(), n, n, np, aa ? -1 : 1, lword, run0, rdelta))
+    if (build_runs(nbr.data(), n, n, np, aa ? -1 : 1, lword, run0, rdelta)) {
         d->n_runs = (int64_t)rdelta.size() / kRunStride;
+        runs_for_device(rdelta, lword, mask.data(), n, ctx->scheme, np);
+    }
     d->io_codes_host = codes;
     d->slot_of_dev.assign(slot_of.begin(), slot_of.end());
     d->slots_host = slots;
@@ -1516,6 +1536,18 @@ int hg_coupling_factors(const int64_t *art_c, const double *art_a, int32_t na, c
 // ================================================================ stepping
 namespace {
 
+// The run-encoded variants (8..14) step only domains that have a run encoding, in a shape
+// of their own; a launch over any other domain takes the table form of the same variant.
+CollideCfg collide_cfg(const hg_ctx *ctx, bool runs, int parity, bool one_domain) {
+    CollideCfg cfg{ctx->storage, ctx->scheme, ctx->block, ctx->spt, ctx->variant};
+    if (cfg.variant >= 8 && !runs)
+        cfg.variant = cfg.variant == 8 || cfg.variant == 12 || cfg.variant == 13 ? 3
+                      : cfg.variant == 9                                      ? 5
+                      : cfg.variant == 10 || cfg.variant == 14                ? 6
+                                                                              : 7;
+    return run_cfg(cfg, parity, one_domain);
+}
+
 int build_plan(hg_ctx *ctx, const std::vector<int32_t> &doms, Plan *&out) {
     PlanKey key{doms};
     auto it = ctx->plans.find(key);
@@ -1525,7 +1557,6 @@ int build_plan(hg_ctx *ctx, const std::vector<int32_t> &doms, Plan *&out) {
     }
     std::unique_ptr<Plan> p(new Plan);
     p->doms = doms;
-    const int64_t ts = (int64_t)ctx->block * ctx->spt;
     std::vector<TileDev> tiles;
     std::vector<IoDev> ios;
     std::vector<int2> chunks;
@@ -1550,6 +1581,10 @@ int build_plan(hg_ctx *ctx, const std::vector<int32_t> &doms, Plan *&out) {
                 ++n_sep;
             }
     }
+    for (size_t j = 0; j < doms.size(); ++j)
+        if (!separate[j]) p->tiles_runs = p->tiles_runs && ctx->doms[doms[j]]->n_runs > 0;
+    const CollideCfg tcfg = collide_cfg(ctx, p->tiles_runs, 0, false);
+    const int64_t ts = (int64_t)tcfg.block * tcfg.spt;  // the same for every parity
     for (size_t j = 0; j < doms.size(); ++j) {
         const int32_t di = doms[j];
         hg_domain *d = ctx->doms[di];
@@ -1557,7 +1592,6 @@ int build_plan(hg_ctx *ctx, const std::vector<int32_t> &doms, Plan *&out) {
             p->sep.push_back(make_domdev(ctx, d));
             p->sep_n.push_back(d->n);
         } else if (doms.size() > 1) {
-            p->tiles_runs = p->tiles_runs && d->n_runs > 0;
             for (int64_t s = 0; s < d->n; s += ts) {
                 TileDev t;
                 t.dom = di;
@@ -1638,9 +1672,6 @@ int build_plan(hg_ctx *ctx, const std::vector<int32_t> &doms, Plan *&out) {
     if (doms.size() == 1) {
         p->single = true;
         p->one = make_domdev(ctx, ctx->doms[doms[0]]);
-        p->tiles_runs = ctx->doms[doms[0]]->n_runs > 0;
-        const int64_t n1 = ctx->doms[doms[0]]->n;
-        p->n_tiles = (n1 + ts - 1) / ts;
     }
     p->n_chunks = (int)chunks.size();
     int rc = dev_alloc(ctx, p->tiles, std::max<size_t>(1, tiles.size()) * sizeof(TileDev));
@@ -1732,35 +1763,26 @@ cudaError_t enqueue_halo(hg_ctx *ctx, Plan *p, int off) {
 // start while the previous step's iolet update runs; separate per-domain launches
 // after the first may start while the previous one runs (they share no data within
 // a step; sites with iolet links still wait, through the chain, for that update).
-// The run-encoded variants (8..11) step only domains that have a run encoding;
-// a launch over any other domain takes the table form of the same variant.
-CollideCfg collide_cfg(hg_ctx *ctx, bool runs) {
-    CollideCfg cfg{ctx->storage, ctx->scheme, ctx->block, ctx->spt, ctx->variant};
-    if (cfg.variant >= 8 && !runs)
-        cfg.variant = cfg.variant == 8 || cfg.variant == 12 || cfg.variant == 13 ? 3
-                      : cfg.variant == 9                                      ? 5
-                      : cfg.variant == 10 || cfg.variant == 14                ? 6
-                                                                              : 7;
-    return cfg;
-}
-
 cudaError_t launch_sc(hg_ctx *ctx, Plan *p, int off, int parity, bool overlap) {
     const int64_t *steps = (const int64_t *)ctx->steps.p;
     const DomDev *table = (const DomDev *)ctx->dom_table.p;
-    const int64_t ts = (int64_t)ctx->block * ctx->spt;
     bool chained = overlap;
-    for (size_t j = 0; j < p->sep.size(); ++j) {
-        if (p->sep_n[j] == 0) continue;
-        const OneDomain one{&p->sep[j], p->sep_n[j], steps, chained};
-        const cudaError_t e = launch_stream_collide(collide_cfg(ctx, p->sep[j].lword != nullptr), table, nullptr,
-                                                    (p->sep_n[j] + ts - 1) / ts, off, parity, one, ctx->stream);
-        if (e != cudaSuccess) return e;
+    auto one_domain = [&](const DomDev &D, int64_t n) {
+        if (n == 0) return cudaSuccess;
+        const CollideCfg cfg = collide_cfg(ctx, D.lword != nullptr, parity, true);
+        const int64_t ts = (int64_t)cfg.block * cfg.spt;
+        const OneDomain one{&D, n, steps, chained};
         chained = true;
+        return launch_stream_collide(cfg, table, nullptr, (n + ts - 1) / ts, off, parity, one, ctx->stream);
+    };
+    for (size_t j = 0; j < p->sep.size(); ++j) {
+        const cudaError_t e = one_domain(p->sep[j], p->sep_n[j]);
+        if (e != cudaSuccess) return e;
     }
+    if (p->single) return one_domain(p->one, ctx->doms[p->doms[0]]->n);
     if (p->n_tiles == 0) return cudaSuccess;
-    const OneDomain one{p->single ? &p->one : nullptr, p->single ? ctx->doms[p->doms[0]]->n : 0, steps, chained};
-    return launch_stream_collide(collide_cfg(ctx, p->tiles_runs), table, (const TileDev *)p->tiles.p, p->n_tiles,
-                                 off, parity, one, ctx->stream);
+    return launch_stream_collide(collide_cfg(ctx, p->tiles_runs, parity, false), table, (const TileDev *)p->tiles.p,
+                                 p->n_tiles, off, parity, OneDomain{nullptr, 0, steps, chained}, ctx->stream);
 }
 
 cudaError_t enqueue_steps(hg_ctx *ctx, Plan *p, int64_t k, int mode) {
@@ -2251,10 +2273,11 @@ int split_plan(hg_split *sp, Plan *&out) {
     }
     std::unique_ptr<Plan> p(new Plan);
     p->doms = key.doms;
-    const int64_t ts = (int64_t)ctx->block * ctx->spt;
+    for (const SplitPart &P : sp->parts) p->tiles_runs = p->tiles_runs && P.n_runs > 0;
+    const CollideCfg tcfg = collide_cfg(ctx, p->tiles_runs, 2, false);
+    const int64_t ts = (int64_t)tcfg.block * tcfg.spt;
     std::vector<TileDev> tiles;
     for (const SplitPart &P : sp->parts) {
-        p->tiles_runs = p->tiles_runs && P.n_runs > 0;
         for (int64_t s = 0; s < P.n_own; s += ts) tiles.push_back(TileDev{P.idx, (int32_t)std::min(ts, P.n_own - s), s});
     }
     std::vector<IoDev> ios;
@@ -2569,6 +2592,7 @@ int hg_split_create(hg_ctx *ctx, const int32_t *xyz, int64_t n, const hg_iolet *
         // owned sites only (ghost rows are never read); entries may point at ghosts
         if (build_runs(T.data(), P.n_own, P.n_loc, np, 1, lw[p], r0[p], rd[p])) {
             P.n_runs = (int64_t)rd[p].size() / kRunStride;
+            runs_for_device(rd[p], lw[p], (const uint32_t *)mask[p].data(), P.n_own, HG_SCHEME_AB, np);
             A(P.lword, lw[p].size() * 4);
             A(P.run0, r0[p].size() * 4);
             A(P.rdelta, rd[p].size() * 4);
@@ -2645,6 +2669,7 @@ int hg_split_create(hg_ctx *ctx, const int32_t *xyz, int64_t n, const hg_iolet *
         D.err = (int32_t *)ctx->errw.p;
         D.n = P.n_loc;
         D.np = P.np;
+        D.neg_zero2 = 0x8000000080000000ull;
         D.omega = (float)(1.0 / tau);
         D.n_io = nio;
         D.slot_site = (const int32_t *)sp->slot_site.p;

@@ -28,11 +28,11 @@ struct DomDev {
     // The same table run-length encoded (null when it does not compress): per site
     // a word whose bits 0..17 flag the non-fluid links (their entry is the virtual
     // index) and whose bits 18..27 give the site's run relative to the run of its
-    // 1024-site chunk (run0); per run the 18 offsets (entry minus site index) its
-    // fluid links share.
+    // 1024-site chunk (run0); per run the 18 offsets its fluid links share.
     const uint32_t *lword;
     const int32_t *run0;
-    const int32_t *rdelta;    // kRunStride entries per run: 18 offsets, 2 zeros (16-byte rows)
+    const int32_t *rdelta;    // kRunStride entries per run: 18 offsets from the own site in the first
+                              // row of the link's opposite pair, 2 zeros (16-byte rows)
     const uint32_t *iomask;   // bit s: site s has an iolet link
     const int32_t *ioprefix;  // per 32-site word: flagged sites before it (slot = rank of the flag)
     const int32_t *io_codes;  // per slot x 18: canonical codes (-1 wall, -(2+k) iolet, >= 0 fluid)
@@ -44,6 +44,7 @@ struct DomDev {
     int32_t *err;             // context error word: set when a bounded device wait gives up
     int64_t n;                // sites
     int64_t np;               // row stride (n padded)
+    unsigned long long neg_zero2;  // the bits of two FP32 -0 (see vmul_apart)
     float omega;              // 1 / tau
     int32_t n_io;
     // read by the body-force pass only (kept after the fields stream-collide reads)
@@ -112,8 +113,27 @@ struct CollideCfg {
                   // 2 = as 1, and the AA even step moves whole rows with TMA bulk copies,
                   // 3 = as 0 with L2 prefetch hints, 4 = as 1 with the AA odd step's
                   // stores staged in shared memory (spt 1), 5 = A/B on adjacent site
-                  // pairs (16-bit storage, spt 2)
+                  // pairs (16-bit storage, spt 2), 6 / 7 = AA on adjacent site pairs (spt 2,
+                  // 7 with hints), 8..14 = the run encoding, in the shape of run_cfg
 };
+
+// Launch shape of the run-encoded kernel.  Measured on the ~10M-site tree (us): FP32 A/B 256 x 2
+// 241, 128 x 2 243, 256 x 1 246, 512 x 2 246; 16-bit A/B 256 x 1 181, 128 x 1 190, 256 x 2 182,
+// 512 x 1 190; AA odd 128 x 1 272 (FP32) and 198 (FP16), 256 x 1 274 and 203, 128 x 2 307 and
+// 236 (64 registers against 40); AA even (site pairs) 128 x 2 225 and 123, 256 x 2 225 and 125.
+// A tile table serves odd and even launches alike: its tiles hold 256 sites.
+constexpr int kRunTile = 256;
+__host__ __device__ constexpr int run_spt(int storage, int scheme, int parity) {
+    return scheme == kAB ? (storage == kF32 ? 2 : 1) : (parity == 1 ? 1 : 2);
+}
+inline CollideCfg run_cfg(CollideCfg cfg, int parity, bool one_domain) {
+    if (cfg.variant < 8) return cfg;
+    cfg.spt = run_spt(cfg.storage, cfg.scheme, parity);
+    cfg.block = kRunTile / cfg.spt;
+    if (one_domain && cfg.scheme == kAB && cfg.storage == kF32) cfg.block = 256;
+    if (one_domain && cfg.scheme == kAA) cfg.block = 128;
+    return cfg;
+}
 
 // parity (AA only): 0 = every domain runs an even step, 1 = odd, 2 = per-domain
 // parity read from the step counters.
