@@ -104,7 +104,8 @@ typedef struct {
     int32_t scheme;           /* HG_SCHEME_* */
     int32_t block_size;       /* stream-collide threads per block (multiple of 32, <= 512); 0 = 256 */
     int32_t sites_per_thread; /* 1, 2 or 4; 0 = 1 */
-    int32_t graph_steps;      /* steps captured per CUDA graph; 0 = 16; negative = no graphs */
+    int32_t graph_steps;      /* steps captured per CUDA graph; 0 = 16; negative = no graphs
+                                 (sets stepped by resident launches use none, see hg_step) */
     int32_t kernel_variant;   /* stream-collide form; every form gives bit-identical results:
                                  0 = gathers into registers;
                                  1 = gathers staged in shared memory by cp.async, AA even step
@@ -319,7 +320,9 @@ int hg_coupling_factors(const int64_t *art_centres, const double *art_areas, int
  * rules on non-fluid links, with boundary values of time t), collides (LBGK,
  * tau) into F_t, then reduces the iolet means of time t in FP64 and sets the
  * boundary values of time t+1 (pulses; coupled inlets from the means).
- * Groups of steps run as captured CUDA graphs.  Asynchronous.
+ * Groups of steps run as captured CUDA graphs; the steps of a small set of
+ * domains (up to 700,000 sites A/B, 450,000 AA, forward coupling) run in
+ * resident launches of up to 1024 steps, with the same bits.  Asynchronous.
  * Passage: Section 2 (the LB step: D3Q19 streaming, LBGK collision, walls,
  * iolets) and Section 2.3 (coupled values exchanged every step). */
 int hg_step(hg_ctx *ctx, int64_t n_steps);

@@ -22,9 +22,11 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 _PARTS = [(s, c, p) for s in (0, 1, 2) for c, p in ((0, 2), (1, 0), (1, 1), (1, 2))]
 UNITS = ([("hg_sc_part.cu", f"hg_sc_{s}{c}{p}", [f"-DHG_PART_S={s}", f"-DHG_PART_SCHEME={c}",
                                                    f"-DHG_PART_PAR={p}"]) for s, c, p in _PARTS]
+         + [("hg_steps.cu", f"hg_steps_{s}{c}", [f"-DHG_PART_S={s}", f"-DHG_PART_SCHEME={c}"])
+            for s in (0, 1, 2) for c in (0, 1)]
          + [("hg_kernels.cu", "hg_kernels", []), ("hg_host.cpp", "hg_host", []), ("hg_noalloc.cu", "hg_noalloc", [])])
 SOURCES = sorted({u[0] for u in UNITS})
-HEADERS = ["hg_internal.h", "hg_device.cuh", os.path.join("..", "..", "include", "hemegb.h")]
+HEADERS = ["hg_internal.h", "hg_device.cuh", "hg_iolet.cuh", "hg_steps.h", os.path.join("..", "..", "include", "hemegb.h")]
 
 
 def _stale() -> bool:

@@ -91,15 +91,15 @@ template <int B, int E, typename F> __device__ __forceinline__ void unroll(F &&f
     }
 }
 
-// Iolet rule for link I of a site next to iolet k (boundary slot `slot`); raw =
-// the site's own post-collision value leaving towards x - c_I (direction opp(I)),
-// in the collision variable.  Scaled storage (h = f~/w) drops the w_I factors
-// (w_I = w_opp(I)); its velocity coefficients are stored divided by w_I.
-template <int I, bool SC>
-__device__ __forceinline__ float iolet_rule(const DomDev &D, const float *bcv, int k, int slot, float raw) {
-    const float val = bcv[k];
-    if (D.io_kind[k] == 0) return -raw + (SC ? 2.0f * val : mulw<I>(2.0f * val));  // anti-bounce-back
-    return __fmaf_rn(val, D.coef[(int64_t)slot * 18 + (I - 1)], raw);       // moving wall
+// Iolet rules for link I of a site next to iolet k; raw = the site's own post-collision value
+// leaving towards x - c_I (direction opp(I)), in the collision variable; val = the iolet's
+// boundary value.  Scaled storage (h = f~/w) drops the w_I factors (w_I = w_opp(I)); its
+// velocity coefficients are stored divided by w_I.
+template <int I, bool SC> __device__ __forceinline__ float pressure_rule(float val, float raw) {
+    return -raw + (SC ? 2.0f * val : mulw<I>(2.0f * val));  // anti-bounce-back
+}
+__device__ __forceinline__ float velocity_rule(float val, float coef, float raw) {
+    return __fmaf_rn(val, coef, raw);  // moving wall
 }
 
 // LBGK collision in deviation form, in place on g[19]; returns (drho, u).
@@ -124,13 +124,13 @@ __device__ __forceinline__ F2 pk2(float a, float b) {
     return r;
 }
 __device__ __forceinline__ float lo2(F2 x) {
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+    float a;
+    asm("{\n\t.reg .f32 t;\n\tmov.b64 {%0, t}, %1;\n\t}" : "=f"(a) : "l"(x.v));
     return a;
 }
 __device__ __forceinline__ float hi2(F2 x) {
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+    float b;
+    asm("{\n\t.reg .f32 t;\n\tmov.b64 {t, %0}, %1;\n\t}" : "=f"(b) : "l"(x.v));
     return b;
 }
 __device__ __forceinline__ float vadd(float a, float b) { return HG_ADD(a, b); }
@@ -369,13 +369,57 @@ __device__ __forceinline__ bool site_flag(const DomDev &D, int64_t s, uint32_t &
 __device__ __forceinline__ int site_slot(const DomDev &D, int64_t s, uint32_t word) {
     return __ldg(D.ioprefix + (s >> 5)) + __popc(word & ((1u << (s & 31)) - 1u));
 }
-template <int S>
-__device__ __forceinline__ void apply_iolet_links(const DomDev &D, const float *bcv, int slot, float g[19]) {
+// f(IC<I>, rule) for every iolet link of boundary slot `slot`, rule: raw value -> value.  A
+// slot whose links all lead into one iolet (nearly every one) has its mask and iolet in one
+// word, so its value and kind are one round of loads, where decoding the 18 codes one after
+// another chained up to three loads per link.  AHEAD also loads the velocity coefficients
+// ahead of the links (18 registers: for the resident kernel, whose steps wait for these).
+template <int S, bool AHEAD, typename F>
+__device__ __forceinline__ void each_iolet_link(const DomDev &D, const float *bcv, int slot, uint32_t word, F &&f) {
+    constexpr bool SC = St<S>::kScaled;
+    const float *coef = D.coef + (int64_t)slot * 18;
+    if (word != kManyIolets) {
+        const int k = (int)(word >> 18);
+        const float val = bcv[k];
+        if (D.io_kind[k] == 0) {
+            unroll<1, 19>([&](auto ic) {
+                constexpr int I = decltype(ic)::v;
+                if ((word >> (I - 1)) & 1u) f(ic, [&](float raw) { return pressure_rule<I, SC>(val, raw); });
+            });
+        } else {
+            float c[18];
+            if constexpr (AHEAD) {
+#pragma unroll
+                for (int i = 0; i < 18; ++i) c[i] = __ldg(coef + i);
+            }
+            unroll<1, 19>([&](auto ic) {
+                constexpr int I = decltype(ic)::v;
+                if ((word >> (I - 1)) & 1u)
+                    f(ic, [&](float raw) {
+                        return velocity_rule(val, AHEAD ? c[I - 1] : __ldg(coef + (I - 1)), raw);
+                    });
+            });
+        }
+        return;
+    }
     const int32_t *codes = D.io_codes + (int64_t)slot * 18;
     unroll<1, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
-        const int32_t c = __ldg(codes + (I - 1));
-        if (c < -1) g[I] = iolet_rule<I, St<S>::kScaled>(D, bcv, -c - 2, slot, g[I]);
+        const int32_t k = -__ldg(codes + (I - 1)) - 2;
+        if (k >= 0)
+            f(ic, [&](float raw) {
+                return D.io_kind[k] == 0 ? pressure_rule<I, SC>(bcv[k], raw)
+                                         : velocity_rule(bcv[k], __ldg(coef + (I - 1)), raw);
+            });
+    });
+}
+__device__ __forceinline__ uint32_t io_word(const DomDev &D, int slot) { return __ldg(D.io_words + slot); }
+template <int S, bool AHEAD = false>
+__device__ __forceinline__ void apply_iolet_links(const DomDev &D, const float *bcv, int slot, uint32_t word,
+                                                  float g[19]) {
+    each_iolet_link<S, AHEAD>(D, bcv, slot, word, [&](auto ic, auto rule) {
+        constexpr int I = decltype(ic)::v;
+        g[I] = rule(g[I]);
     });
 }
 // A stream-collide launch may start while the previous step's iolet update is
@@ -394,20 +438,16 @@ __device__ __forceinline__ int iolet_fixup(const DomDev &D, int64_t s, float g[1
     if (!site_flag(D, s, word)) return -1;
     wait_for_iolet_update();
     const int slot = site_slot(D, s, word);
-    apply_iolet_links<S>(D, D.bcv, slot, g);
+    apply_iolet_links<S>(D, D.bcv, slot, io_word(D, slot), g);
     return slot;
 }
 // The same for one half of a packed pair (HI: the second site); the caller found the flag.
 template <int S, bool HI>
 __device__ __forceinline__ void iolet_links_half(const DomDev &D, const float *bcv, int slot, F2 g[19]) {
-    const int32_t *codes = D.io_codes + (int64_t)slot * 18;
-    unroll<1, 19>([&](auto ic) {
+    each_iolet_link<S, false>(D, bcv, slot, io_word(D, slot), [&](auto ic, auto rule) {
         constexpr int I = decltype(ic)::v;
-        const int32_t c = __ldg(codes + (I - 1));
-        if (c < -1) {
-            const float v = iolet_rule<I, St<S>::kScaled>(D, bcv, -c - 2, slot, HI ? hi2(g[I]) : lo2(g[I]));
-            g[I] = HI ? pk2(lo2(g[I]), v) : pk2(v, hi2(g[I]));
-        }
+        const float a = lo2(g[I]), b = hi2(g[I]);
+        g[I] = HI ? pk2(a, rule(b)) : pk2(rule(a), b);
     });
 }
 template <int S>
@@ -904,7 +944,7 @@ __device__ __forceinline__ void site_run(const DomDev &D, const typename St<S>::
     if (r.w >> 31) {  // a link into an iolet opening
         wait_for_iolet_update();
         slot = site_slot(D, s, __ldg(D.iomask + (s >> 5)));
-        apply_iolet_links<S>(D, D.bcv, slot, g);
+        apply_iolet_links<S>(D, D.bcv, slot, io_word(D, slot), g);
     }
     const float4 m = collide_s<S>(g, D.omega);
     int32_t *back = stash;

@@ -33,6 +33,7 @@
 
 #include "../../include/hemegb.h"
 #include "hg_internal.h"
+#include "hg_steps.h"
 
 using namespace hg;
 
@@ -466,6 +467,12 @@ struct Plan {
     int n_fslots = 0;  // (domain, slot) pairs the body-force pass visits
     int n_ios = 0;
     int n_chunks = 0;
+    // resident multi-step launches (hg_steps.cu): tables and buffers of the set, made
+    // on first use; 0 = not looked at yet, 1 = ready, -1 = the set is stepped launch by launch
+    int resident = 0;
+    DevBuf res;
+    StepsArgs res_args{};
+    StepsShape res_shape;
     cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};  // by parity mode
     int graph_steps = 0;
 };
@@ -622,10 +629,29 @@ void drop_plans(hg_ctx *ctx) {
         for (auto &g : p.graph)
             if (g) cudaGraphExecDestroy(g);
         for (DevBuf *b : {&p.tiles, &p.ios, &p.adv, &p.chunks, &p.partials, &p.counters, &p.rev, &p.fslots,
-                          &p.halo_pack, &p.halo_unpack, &p.send, &p.recv, &p.halo_moves})
+                          &p.halo_pack, &p.halo_unpack, &p.send, &p.recv, &p.halo_moves, &p.res})
             dev_free(ctx, *b);
     }
     ctx->plans.clear();
+}
+
+// Appends DomDev::io_words (one per boundary slot) to the slots' 18 link codes.
+void append_io_words(std::vector<int32_t> &codes) {
+    const size_t n = codes.size() / 18;
+    codes.resize(n * 19);
+    for (size_t sl = 0; sl < n; ++sl) {
+        uint32_t word = 0;
+        int32_t iolet = -1;
+        bool many = false;
+        for (int i = 0; i < 18; ++i) {
+            const int32_t k = -codes[sl * 18 + i] - 2;
+            if (k < 0) continue;
+            many = many || (iolet >= 0 && iolet != k);
+            iolet = k;
+            word |= 1u << i;
+        }
+        codes[n * 18 + sl] = (int32_t)(many ? kManyIolets : word | (uint32_t)std::max(0, iolet) << 18);
+    }
 }
 
 DomDev make_domdev(hg_ctx *ctx, hg_domain *d) {
@@ -640,6 +666,7 @@ DomDev make_domdev(hg_ctx *ctx, hg_domain *d) {
     D.iomask = (const uint32_t *)d->iomask.p;
     D.ioprefix = (const int32_t *)d->ioprefix.p;
     D.io_codes = (const int32_t *)d->io_codes.p;
+    D.io_words = (const uint32_t *)(D.io_codes + 18 * std::max<int64_t>(1, d->n_adj));
     D.slot_site = (const int32_t *)d->slot_site.p;
     D.bnd = (float4 *)d->bnd.p;
     D.coef = (const float *)d->coef.p;
@@ -1185,6 +1212,7 @@ int hg_domain_create(hg_ctx *ctx, const int32_t *xyz, int64_t n, const hg_iolet 
         runs_for_device(rdelta, lword, mask.data(), n, ctx->scheme, np);
     }
     d->io_codes_host = codes;
+    append_io_words(codes);
     d->slot_of_dev.assign(slot_of.begin(), slot_of.end());
     d->slots_host = slots;
     d->canon_of_host = canon_of;
@@ -1826,9 +1854,189 @@ int ensure_graph(hg_ctx *ctx, Plan *p, int mode) {
     return HG_OK;
 }
 
-// n steps of a plan: whole groups as graph replays, the rest launched directly.
+// ---- resident multi-step launches ----
+cudaError_t steps_blocks(const hg_ctx *ctx, bool stash, int threads, size_t smem, int *out) {
+#define HG_CASE(S_, C_) \
+    if (ctx->storage == S_ && ctx->scheme == C_) return steps_blocks_per_sm<S_, C_>(stash, threads, smem, out);
+    HG_CASE(0, 0) HG_CASE(0, 1) HG_CASE(1, 0) HG_CASE(1, 1) HG_CASE(2, 0) HG_CASE(2, 1)
+#undef HG_CASE
+    return cudaErrorInvalidValue;
+}
+cudaError_t steps_launch(const hg_ctx *ctx, const StepsArgs &a, const StepsShape &sh) {
+#define HG_CASE(S_, C_) \
+    if (ctx->storage == S_ && ctx->scheme == C_) return launch_steps<S_, C_>(a, sh, ctx->stream);
+    HG_CASE(0, 0) HG_CASE(0, 1) HG_CASE(1, 0) HG_CASE(1, 1) HG_CASE(2, 0) HG_CASE(2, 1)
+#undef HG_CASE
+    return cudaErrorInvalidValue;
+}
+
+// Largest set (sites of all its domains) that is stepped by resident launches.  Time per step of
+// a tree of n sites, launch by launch / resident (us; the slower of Morton and rows ordering
+// against its resident time): 290k FP32 A/B 16.7 / 8.9, FP16 AA 17.9 / 10.9; 385k FP32 A/B
+// 17.7 / 10.7, FP16 AA 19.5 / 17.4 (links no longer fit shared memory with three blocks per
+// SM); 480k FP16 AA 19.8 / 22.0, FP32 AA 21.1 / 23.2; 630k FP32 A/B 23.3 / 19.2, FP16 A/B
+// 17.3 / 15.7; 770k FP32 A/B 26.8 / 26.7, FP16 A/B 18.2 / 18.3.
+int64_t resident_sites(const hg_ctx *ctx) { return ctx->scheme == HG_SCHEME_AB ? 700000 : 450000; }
+
+// The shape of a resident launch over domains of the given sizes; false: none fits.  The
+// smallest blocks that give every block one tile, else the fewest tiles per block.
+bool steps_shape(const hg_ctx *ctx, const std::vector<int64_t> &sizes, int n_ios, StepsShape &sh, int &n_site_blocks) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return false;
+    // iolet blocks: up to a sixth of the SMs' worth, one iolet each where that is enough, and
+    // then up to three blocks per iolet taking its steps in turn
+    const int sets = std::max((n_ios + kStepsIolets - 1) / kStepsIolets, std::min(n_ios, sms / 6));
+    sh.groups = sets == 0 ? 1 : std::max(1, std::min(kStepsLag - 1, sms / 6 / sets));
+    const int n_io = sets * sh.groups;
+    for (int own = 1; own <= kStepsTiles; ++own)
+        for (int threads = own == 1 ? 128 : kStepsThreads; threads <= kStepsThreads; threads *= 2) {
+            int64_t tiles = 0;
+            for (int64_t n : sizes) tiles += (n + threads - 1) / threads;
+            n_site_blocks = (int)((tiles + own - 1) / own);
+            for (const bool stash : {true, false}) {
+                const size_t smem = stash ? (size_t)own * kStashRows * 4 * threads : 0;
+                int per_sm = 0;
+                if (smem > 200 * 1024) continue;
+                if (steps_blocks(ctx, stash, threads, smem, &per_sm) != cudaSuccess) {
+                    cudaGetLastError();
+                    return false;
+                }
+                // small blocks: spread over the SMs rather than stacked on a few
+                const int64_t room = (int64_t)sms * std::min(per_sm, threads < kStepsThreads ? 2 : kStepsPerSm);
+                if (n_site_blocks + n_io > room) continue;
+                sh.threads = threads;
+                sh.smem = smem;
+                sh.stash = stash;
+                sh.grid = n_site_blocks + n_io;
+                return true;
+            }
+        }
+    return false;
+}
+
+// Tables of a resident launch; leaves p->resident at 1, or -1 where the set does not qualify.
+int ensure_resident(hg_ctx *ctx, Plan *p) {
+    if (p->resident != 0) return HG_OK;
+    p->resident = -1;
+    if (ctx->couple_mode != HG_COUPLE_FORWARD || p->n_fslots > 0 || p->n_halo > 0) return HG_OK;
+    std::vector<hg_domain *> doms;
+    std::vector<int64_t> sizes;
+    int64_t total = 0;
+    std::map<int32_t, int32_t> at;  // context index -> place in the set
+    for (int32_t di : p->doms) {
+        hg_domain *d = di < (int32_t)ctx->doms.size() ? ctx->doms[di] : nullptr;
+        if (!d) return HG_OK;  // a split's partitions
+        at[di] = (int32_t)doms.size();
+        doms.push_back(d);
+        sizes.push_back(d->n);
+        total += d->n;
+        if (19 * d->np > INT32_MAX) return HG_OK;  // links are 32-bit element indices
+    }
+    if (total == 0 || total > resident_sites(ctx)) return HG_OK;
+    StepsShape sh;
+    int n_site_blocks = 0;
+    if (!steps_shape(ctx, sizes, p->n_ios, sh, n_site_blocks)) return HG_OK;
+    std::vector<StepsDom> sd(doms.size());
+    std::vector<TileDev> tiles;
+    std::vector<StepsIo> sios;
+    std::vector<StepsFed> fed;
+    int n_sources = 0;
+    size_t alt = 0;  // bytes of the boundary values and moments of several steps
+    auto pad = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    for (size_t j = 0; j < doms.size(); ++j) {
+        hg_domain *d = doms[j];
+        for (int64_t s = 0; s < d->n; s += sh.threads)
+            tiles.push_back(TileDev{(int32_t)j, (int32_t)std::min<int64_t>(sh.threads, d->n - s), s});
+        sd[j].D = make_domdev(ctx, d);
+        sd[j].coupled = 0;
+        sd[j].n_adj = d->n_adj;
+        sd[j].values = (float *)alt;  // offsets for now
+        alt += pad((size_t)d->nio * 4 * kStepsMax);
+        sd[j].moments = (float4 *)alt;
+        alt += pad((size_t)d->n_adj * 16 * kStepsLag);
+    }
+    {
+        std::lock_guard<std::mutex> lk(ctx->mu);
+        for (size_t j = 0; j < doms.size(); ++j)
+            for (int k = 0; k < doms[j]->nio; ++k) {
+                StepsIo q{(int32_t)j, k, (int32_t)fed.size(), 0};
+                for (const auto &c : ctx->coupled)
+                    if (c.second.src_dom == doms[j]->idx && c.second.src_k == k && at.count(c.first.first)) {
+                        fed.push_back(StepsFed{at[c.first.first], c.first.second, c.second.factor});
+                        sd[at[c.first.first]].coupled = 1;
+                    }
+                q.n_fed = (int32_t)fed.size() - q.fed0;
+                n_sources += q.n_fed > 0;
+                sios.push_back(q);
+            }
+    }
+    if ((int)sios.size() != p->n_ios) return HG_OK;
+    const size_t b_sync = pad(sizeof(StepsSync)), b_dom = pad(sd.size() * sizeof(StepsDom)),
+                 b_tile = pad(tiles.size() * sizeof(TileDev)), b_io = pad(sios.size() * sizeof(StepsIo)),
+                 b_fed = pad(fed.size() * sizeof(StepsFed));
+    const size_t b_tab = b_sync + b_dom + b_tile + b_io + b_fed;
+    if (dev_alloc(ctx, p->res, b_tab + alt) != HG_OK) {
+        cudaGetLastError();
+        return HG_OK;  // no room: launch by launch
+    }
+    char *base = (char *)p->res.p;
+    for (StepsDom &d : sd) {
+        d.values = (float *)(base + b_tab + (size_t)d.values);
+        d.moments = (float4 *)(base + b_tab + (size_t)d.moments);
+    }
+    std::vector<char> up(b_tab, 0);
+    char *u = up.data() + b_sync;
+    memcpy(u, sd.data(), sd.size() * sizeof(StepsDom));
+    memcpy(u += b_dom, tiles.data(), tiles.size() * sizeof(TileDev));
+    if (!sios.empty()) memcpy(u + b_tile, sios.data(), sios.size() * sizeof(StepsIo));
+    if (!fed.empty()) memcpy(u + b_tile + b_io, fed.data(), fed.size() * sizeof(StepsFed));
+    // stream-ordered before the first launch (a pageable source is staged on the call)
+    CU(ctx, cudaMemcpyAsync(base, up.data(), b_tab, cudaMemcpyHostToDevice, ctx->stream));
+    StepsArgs &a = p->res_args;
+    a.sync = (StepsSync *)base;
+    a.doms = (const StepsDom *)(base + b_sync);
+    a.tiles = (const TileDev *)(base + b_sync + b_dom);
+    a.sios = (const StepsIo *)(base + b_sync + b_dom + b_tile);
+    a.fed = (const StepsFed *)(base + b_sync + b_dom + b_tile + b_io);
+    a.ios = (const IoDev *)p->ios.p;
+    a.err = (int32_t *)ctx->errw.p;
+    a.n_doms = (int32_t)sd.size();
+    a.n_tiles = (int32_t)tiles.size();
+    a.n_ios = p->n_ios;
+    a.n_sources = n_sources;
+    a.n_site_blocks = n_site_blocks;
+    a.n_groups = sh.groups;
+    a.stash_words = (int32_t)(sh.smem / 4);
+    p->res_shape = sh;
+    p->resident = 1;
+    return HG_OK;
+}
+
+// n steps of a plan by resident launches; `left` of them remain where it has none.
+int run_resident(hg_ctx *ctx, Plan *p, int64_t n, int64_t &left) {
+    left = n;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return HG_OK;  // a caller's capture records plain launches
+    }
+    const int rc = ensure_resident(ctx, p);
+    if (rc != HG_OK || p->resident != 1) return rc;
+    for (; left > 0; left -= p->res_args.n_steps) {
+        p->res_args.n_steps = (int32_t)std::min<int64_t>(left, kStepsMax);
+        CU(ctx, steps_launch(ctx, p->res_args, p->res_shape));
+    }
+    return HG_OK;
+}
+
+// n steps of a plan: resident launches where the set is small, else whole groups as graph
+// replays and the rest launched directly.
 int run_plan(hg_ctx *ctx, Plan *p, int64_t n, int mode) {
     int64_t left = n;
+    const int rc = run_resident(ctx, p, n, left);
+    if (rc != HG_OK) return rc;
+    if (mode != 2) mode = (int)((mode + n - left) & 1);
+    n = left;
     if (ctx->graph_steps > 0 && n >= ctx->graph_steps) {
         while (left >= ctx->graph_steps) {
             const int rc = ensure_graph(ctx, p, mode);
@@ -2534,6 +2742,7 @@ int hg_split_create(hg_ctx *ctx, const int32_t *xyz, int64_t n, const hg_iolet *
         if (rc == HG_OK) rc = dev_alloc(ctx, b, bytes);
     };
     A(sp->bnd, (size_t)std::max<int64_t>(1, n_adj) * 16);
+    append_io_words(codes);
     A(sp->io_codes, codes.size() * 4);
     A(sp->coef, coef.size() * 4);
     A(sp->slot_site, slot_site.size() * 4);
@@ -2661,6 +2870,7 @@ int hg_split_create(hg_ctx *ctx, const int32_t *xyz, int64_t n, const hg_iolet *
         D.iomask = (const uint32_t *)P.iomask.p;
         D.ioprefix = (const int32_t *)P.ioprefix.p;
         D.io_codes = (const int32_t *)sp->io_codes.p;
+        D.io_words = (const uint32_t *)(D.io_codes + 18 * std::max<int64_t>(1, sp->n_adj));
         D.bnd = (float4 *)sp->bnd.p;
         D.coef = (const float *)sp->coef.p;
         D.bcv = (const float *)sp->bcv.p;

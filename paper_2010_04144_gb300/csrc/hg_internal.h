@@ -15,6 +15,7 @@ namespace hg {
 // Virtual indices lie outside [0, n).  Links into iolet openings are told apart
 // through iomask / ioprefix / io_codes (canonical codes per boundary slot).
 constexpr int kMaxIolets = 4096;
+constexpr uint32_t kManyIolets = 0xffffffffu;  // a boundary slot whose links lead into several iolets
 
 enum Storage : int { kF32 = 0, kF16 = 1, kBF16 = 2 };
 enum Scheme : int { kAB = 0, kAA = 1 };
@@ -36,6 +37,7 @@ struct DomDev {
     const uint32_t *iomask;   // bit s: site s has an iolet link
     const int32_t *ioprefix;  // per 32-site word: flagged sites before it (slot = rank of the flag)
     const int32_t *io_codes;  // per slot x 18: canonical codes (-1 wall, -(2+k) iolet, >= 0 fluid)
+    const uint32_t *io_words; // per slot: its iolet links (bits 0..17) and their iolet, or kManyIolets
     float4 *bnd;              // per adjacent slot: (drho, ux, uy, uz) of the step's G_t
     const float *coef;        // per adjacent slot x 18: velocity-link coefficient 6 w_i c_i.(-a) phi
     const float *bcv;         // per iolet: boundary value of the step being run

@@ -33,6 +33,7 @@
 // opposite slot -- the bounce-back value -- with no branch.  Links into iolet
 // openings are fixed up on a rare path (iomask, ioprefix, io_codes).
 #include "hg_device.cuh"
+#include "hg_iolet.cuh"
 
 namespace hg {
 namespace {
@@ -40,11 +41,7 @@ namespace {
 // ---- iolet update: FP64 means in fixed order, next boundary value ----
 __device__ __forceinline__ void block_sum2(double &a, double &b) {
     __shared__ double sa[32], sb[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
+    warp_sum2(a, b);
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     __syncthreads();
     if (l == 0) {
@@ -56,11 +53,7 @@ __device__ __forceinline__ void block_sum2(double &a, double &b) {
     if (w == 0) {
         a = l < nw ? sa[l] : 0.0;
         b = l < nw ? sb[l] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            b += __shfl_down_sync(0xffffffffu, b, o);
-        }
+        warp_sum2(a, b);
     }
 }
 
@@ -83,9 +76,7 @@ __global__ void __launch_bounds__(kIoChunk) k_iolet_update(const IoDev *__restri
     double su = 0.0, sr = 0.0;
     const int j = ck.y * kIoChunk + threadIdx.x;
     if (j < I.n_slots) {
-        const float4 m = I.bnd[__ldg(I.slots + j)];
-        su = (double)m.y * I.nx + (double)m.z * I.ny + (double)m.w * I.nz;
-        sr = (double)m.x;
+        iolet_terms(I, I.bnd[__ldg(I.slots + j)], su, sr);
     }
     block_sum2(su, sr);
     if (threadIdx.x == 0) {
@@ -112,10 +103,7 @@ __global__ void __launch_bounds__(kIoChunk) k_iolet_update(const IoDev *__restri
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        const double cnt = (double)I.n_slots;
-        I.M[0] = I.n_slots ? a / cnt : 0.0;
-        I.M[1] = I.n_slots ? b / cnt : 0.0;
-        I.M[2] = cnt;
+        iolet_store_means(I, iolet_mean(I, a), b);
         counters[ck.x] = 0u;
         __threadfence();
         s_last = atomicAdd(&counters[n_ios], 1u) == (unsigned)(n_ios - 1);
@@ -131,14 +119,7 @@ __global__ void __launch_bounds__(kIoChunk) k_iolet_update(const IoDev *__restri
         if (J.coupled) {
             if (forward) *J.bcv = (float)(J.factor * __ldcg(J.src_M));
         } else {
-            // phase of the next step in [0, 1): exact remainder first, so the FP64
-            // cosine only ever sees an argument in [0, 2 pi)
-            const double tn = (double)(e + 1);
-            const double ph = J.pulse ? fmod(tn, J.period) / J.period : 0.0;
-            double p = 1.0;
-            if (J.pulse == 1) p = 0.5 * (1.0 - cos(2.0 * 3.141592653589793 * ph));
-            else if (J.pulse == 2) p = sin(2.0 * 3.141592653589793 * ph);
-            *J.bcv = (float)(J.value * p);
+            *J.bcv = iolet_value(J, e);
         }
         if (!forward && J.n_rev > 0) {
             // reverse: mean over the fed inlets of inflow speed / factor; the outlet's force

@@ -49,7 +49,7 @@ def footprint_bytes(n_sites, storage, scheme, n_iolets=2, iolet_radii=None, reor
     """Upper bound on the HBM bytes of one domain before it is built: distributions,
     neighbour table, iolet mask and prefix per site; the table's run encoding where it is
     built (4 bytes per site plus at most 16 bytes per site of run offsets); moments, link
-    codes, link coefficients and site index per boundary slot (164 B) plus one list entry
+    codes, link coefficients and site index per boundary slot (168 B) plus one list entry
     per (site, iolet) pair; per-iolet values; the two site permutations of a reordered
     layout; and the 256-byte rounding of each buffer.  With the iolet radii the boundary slots are bounded per iolet
     (adjacent_bound); without them 5% of the sites is assumed."""
@@ -62,7 +62,7 @@ def footprint_bytes(n_sites, storage, scheme, n_iolets=2, iolet_radii=None, reor
         n_iolets = len(iolet_radii)
     else:
         adjacent = pairs = 0.05 * n_sites
-    return int(per_site * np_ + 164 * adjacent + 4 * pairs + 64 * n_iolets + 20 * 256 + 4 * 4096)
+    return int(per_site * np_ + 168 * adjacent + 4 * pairs + 64 * n_iolets + 20 * 256 + 4 * 4096)
 
 
 def geometry_footprint(geo, storage, scheme, reordered=False):
