@@ -42,13 +42,13 @@ ORDERINGS = ("morton", "rows", "bricks")
 def bytes_per_update(storage, scheme, variant=0, n=1, n_runs=0):
     """Algorithmic bytes per site update of the stream-collide kernel: the 19 populations
     read and written once each, plus the neighbour table on pull steps (every A/B step, the
-    odd AA steps): its 18 rows (72 bytes), or for the run-encoded variants (8..11, on a
-    domain that has runs) the per-site word (4 bytes), the 80-byte offset rows of the runs
-    shared by their sites and the per-1024-site chunk word.  With the table: 224 / 188 bytes
+    odd AA steps): its 18 rows (72 bytes), or on a domain that has runs (the library then
+    reads those, whatever the variant) the per-site word (4 bytes), the 80-byte offset rows
+    of the runs shared by their sites and the per-1024-site chunk word.  With the table: 224 / 188 bytes
     (FP32 A/B / AA), 148 / 112 (16-bit)."""
     eb = 4 if storage == "f32" else 2
     data = 19 * eb * 2
-    table = 4 + 80 * n_runs / n + 4 / 1024 if (variant >= 8 and n_runs > 0) else 72
+    table = 4 + 80 * n_runs / n + 4 / 1024 if n_runs > 0 else 72
     return data + (table if scheme == "ab" else table / 2)
 
 

@@ -102,35 +102,19 @@ typedef struct {
     int32_t device;           /* CUDA device ordinal */
     int32_t storage;          /* HG_STORE_* */
     int32_t scheme;           /* HG_SCHEME_* */
-    int32_t block_size;       /* stream-collide threads per block (multiple of 32, <= 512); 0 = 256 */
-    int32_t sites_per_thread; /* 1, 2 or 4; 0 = 1 */
+    int32_t block_size;       /* multiple of 32, <= 512; 0 = 256 (see kernel_variant) */
+    int32_t sites_per_thread; /* 1, 2 or 4; 0 = 1 (see kernel_variant) */
     int32_t graph_steps;      /* steps captured per CUDA graph; 0 = 16; negative = no graphs
                                  (sets stepped by resident launches use none, see hg_step) */
-    int32_t kernel_variant;   /* stream-collide form; every form gives bit-identical results:
-                                 0 = gathers into registers;
-                                 1 = gathers staged in shared memory by cp.async, AA even step
-                                     on site pairs (sites_per_thread 1 or 2);
-                                 2 = 1, with the AA even step moved by TMA bulk copies (AA only,
-                                     sites_per_thread 1 or 2);
-                                 3 = 0, with L2 256-byte prefetch hints on every load;
-                                 4 = 1, with the AA odd step's stores staged in shared memory
-                                     and written coalesced (AA only, sites_per_thread 1);
-                                 5 = 0 on pairs of adjacent sites sharing table loads and
-                                     packed stores (A/B with FP16/BF16 storage,
-                                     sites_per_thread 2);
-                                 6 = AA on pairs of adjacent sites: shared table loads for
-                                     the gathers and the scatter, packed rest values, the
-                                     even step on vector pairs (sites_per_thread 2);
-                                 7 = 6 with L2 256-byte prefetch hints on the loads;
-                                 8..14 = one kernel that reads the run-encoded neighbour
-                                     table (hg_domain_runs) instead of the 18 table
-                                     rows, in a launch shape of its own; a launch over
-                                     a domain without a run encoding runs variant 3
-                                     (8, 12, 13), 5 (9), 6 (10, 14) or 7 (11) in the
-                                     shape given.  The shapes accepted with them: any
-                                     (8); those of 5 (9), of 6 (10, 11, 14); 1 or 2
-                                     sites per thread, AA (12); 2 or 4 sites per
-                                     thread (13) */
+    int32_t kernel_variant;   /* 0..14, accepted as before; every one gives the same bits.  The
+                                 stream-collide kernel and its launch shape are the library's
+                                 choice: the run-encoded form on domains that have a run
+                                 encoding (hg_domain_runs), else the 18-row table's, each in
+                                 the shape measured best, whatever the variant, block size and
+                                 sites per thread given.  Accepted together: 0, 3, 8 with any
+                                 sites per thread; 1 with 1 or 2; 2 and 12 with 1 or 2 (AA
+                                 only); 4 with 1 (AA only); 5 and 9 with 2 (A/B, FP16/BF16
+                                 only); 6, 7, 10, 11, 14 with 2 (AA only); 13 with 2 or 4 */
     void *stream;             /* cudaStream_t to order work on; NULL = a stream the context creates */
     hg_alloc_fn alloc;        /* NULL = cudaMalloc */
     hg_free_fn free;          /* NULL = cudaFree */
@@ -228,7 +212,7 @@ int hg_domain_info(hg_domain *d, int64_t *n_sites, int32_t *n_iolets, int64_t *n
  * span starting a new run), plus a 4-byte word per site flagging its non-fluid
  * links.  In rows ordering a run covers most of an x-row of a vessel, so the
  * encoding costs about 4 + 80 / run-length bytes per site (80-byte rows).
- * Kernel variants 8..14 read it; the results are the same bits.
+ * Where it is built the stepping kernels read it; the results are the same bits.
  * Passage: Section 2.2 (indirect addressing of the sparse fluid-site list). */
 int hg_domain_runs(hg_domain *d, int64_t *n_runs);
 
@@ -341,10 +325,10 @@ int hg_step_domains(hg_ctx *ctx, hg_domain *const *doms, int32_t n_doms, int64_t
 int hg_step_profiled(hg_ctx *ctx, int64_t n_steps, double *ms_stream_collide,
                      double *ms_iolet, float *per_step);
 
-/* Change the stream-collide launch shape of an existing context (threads per
- * block: multiple of 32, <= 512; sites per thread: 1, 2 or 4; kernel variant
- * as in hg_ctx_params).  Results do not depend on it (each site's arithmetic
- * is the same); used by the autotuner.  Errors: HG_ERR_ARG.
+/* Change the launch shape recorded for an existing context (threads per block:
+ * multiple of 32, <= 512; sites per thread: 1, 2 or 4; kernel variant as in
+ * hg_ctx_params, which says what it decides).  Results do not depend on it.
+ * Errors: HG_ERR_ARG.
  * Passage: infrastructure: no passage. */
 int hg_ctx_set_launch(hg_ctx *ctx, int32_t block_size, int32_t sites_per_thread,
                       int32_t kernel_variant);

@@ -5,7 +5,9 @@ the context's own domains with CUDA events around every stream-collide launch
 (hg_step_profiled), keeps the fastest, and restores every domain's state, step
 count, boundary values and iolet means afterwards (hg_save_state /
 hg_load_state), so tuning never changes the simulation.  Every candidate
-computes bit-identical results; only the time differs.
+computes bit-identical results.  The library itself picks the kernel form and launch shape a
+launch takes (see kernel_variant in hemegb.h), so the candidates of one context time alike;
+the site ordering is what tuning decides.
 
 Results are kept in a JSON cache (``$HEMEGB_TUNE_CACHE``, default
 ``~/.cache/hemegb/tune.json``) keyed by device, storage, scheme, domain sizes
@@ -25,13 +27,11 @@ DEFAULT_CANDIDATES = (
     (128, 2, 2), (256, 2, 2), (256, 1, 2),  # variant 2: AA scheme only
     (256, 1, 3), (128, 1, 3), (256, 2, 3), (128, 2, 3), (512, 2, 3), (128, 4, 3), (256, 4, 3),
     (128, 2, 5), (256, 2, 5), (512, 2, 5),  # variant 5: A/B with 16-bit storage only
-    (128, 2, 6), (256, 2, 6), (256, 2, 7), (512, 2, 7),  # variants 6, 7: AA on site pairs
+    (128, 2, 6), (256, 2, 6), (256, 2, 7), (512, 2, 7),  # variants 6, 7: AA only
     # 8..14: the run-encoded neighbour table, one kernel in a shape of its own; on domains
     # without one they are 3, 5, 6 and 7 in the shape given
     (256, 1, 8), (256, 2, 9), (256, 2, 10), (256, 2, 11), (128, 1, 12), (128, 2, 13), (128, 2, 14),
 )
-# Variant 4 (staged AA odd-step stores) is measured slower than variant 1 on
-# every workload tried; it stays available through Context.set_launch.
 AA_ONLY = (2, 4, 6, 7, 10, 11, 12, 14)
 AB_16BIT_ONLY = (5, 9)
 

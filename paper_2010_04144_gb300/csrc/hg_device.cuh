@@ -309,19 +309,10 @@ template <bool HINT, typename T> __device__ __forceinline__ T load_rw(const T *p
     else return *p;
 }
 
-// ---- neighbour entries of a site: the 18-row table or its run encoding ----
+// ---- the links of a site: the 18-row neighbour table or its run encoding ----
 // The table (72 bytes per site) gives for link I (1..18) the fluid neighbour's device
 // index, or for a non-fluid link the virtual index s + dd np with dd = opp(I) - I (A/B)
 // or I - opp(I) (AA).
-template <bool HINT> struct TabNb {
-    const int32_t *p;
-    int64_t np;
-    __device__ __forceinline__ TabNb(const DomDev &D, int64_t s) : p(D.nbr + s), np(D.np) {}
-    __device__ __forceinline__ void all(int32_t nb[18]) const {
-#pragma unroll
-        for (int i = 0; i < 18; ++i) nb[i] = load_nbr<HINT>(p + (int64_t)i * np);
-    }
-};
 // The run encoding: a word per site (non-fluid flags, run within the chunk), the
 // chunk's first run, and the run's 80-byte row, which the run's other sites also read
 // (L1 hits): about 4 + 80 / run-length bytes per site.  Rows 2k+1 and 2k+2 of the
@@ -475,41 +466,16 @@ template <typename T> __device__ __forceinline__ T *opaque(T *p) {
     return q;
 }
 
-// ---- A/B pull: F_{t-1} in src, F_t to dst (18-row table) ----
-template <int S, bool HINT = false>
-__device__ __forceinline__ void site_ab(const DomDev &D, const typename St<S>::T *__restrict__ src,
-                                        typename St<S>::T *__restrict__ dst, int64_t s) {
-    using Tr = St<S>;
-    const int64_t np = D.np;
-    int32_t nb[18];
-    TabNb<HINT>(D, s).all(nb);
-    float g[19];
-    g[0] = Tr::template ld<0>(load_ro<HINT>(src + s));
-    unroll<1, 19>([&](auto ic) {  // virtual indices: walls read their own opposite value
-        constexpr int I = decltype(ic)::v;
-        g[I] = Tr::template ld<I>(load_ro<HINT>(src + ((int64_t)I * np + nb[I - 1])));
-    });
-    const int slot = iolet_fixup<S>(D, s, g);
-    const float4 m = collide_s<S>(g, D.omega);
-    unroll<0, 19>([&](auto ic) {
-        constexpr int I = decltype(ic)::v;
-        dst[(int64_t)I * np + s] = Tr::template st<I>(g[I]);
-    });
-    if (slot >= 0) D.bnd[slot] = m;
-}
-
 // ---- AA even step: state G_t natural at the own site -> F_t swapped at the own site ----
-// The store base is passed through an opaque move so the compiler recomputes
-// the 19 store addresses after the collision instead of keeping the load
-// addresses alive across it (75 -> ~45 registers).
-template <int S, bool HINT = false>
+// One site (the ragged end of a tile; the rest goes in pairs).
+template <int S>
 __device__ __forceinline__ void site_aa_even(const DomDev &D, typename St<S>::T *buf, int64_t s) {
     using Tr = St<S>;
     const int64_t np = D.np;
     float g[19];
     unroll<0, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
-        g[I] = Tr::template ld<I>(load_rw<HINT>(buf + (int64_t)I * np + s));
+        g[I] = Tr::template ld<I>(buf[(int64_t)I * np + s]);
     });
     const int slot = iolet_fixup<S>(D, s, g);  // the odd step left raw values on iolet links
     const float4 m = collide_s<S>(g, D.omega);
@@ -521,237 +487,7 @@ __device__ __forceinline__ void site_aa_even(const DomDev &D, typename St<S>::T 
     if (slot >= 0) D.bnd[slot] = m;
 }
 
-// ---- AA odd step: gather F_{t-1} (swapped) from x - c_i, scatter F_t to x + c_i ----
-// Entry OPP(I) of the site's row is the site at x + c_I; its virtual index for
-// a non-fluid link turns the scatter into the raw write to the own slot OPP(I).
-template <int S, bool HINT = false>
-__device__ __forceinline__ void site_aa_odd(const DomDev &D, typename St<S>::T *buf, int64_t s) {
-    using Tr = St<S>;
-    const int64_t np = D.np;
-    int32_t nb[18];
-    TabNb<HINT>(D, s).all(nb);
-    float g[19];
-    g[0] = Tr::template ld<0>(load_rw<HINT>(buf + s));
-    unroll<1, 19>([&](auto ic) {
-        constexpr int I = decltype(ic)::v;
-        g[I] = Tr::template ld<I>(load_rw<HINT>(buf + ((int64_t)OPP(I) * np + nb[I - 1])));
-    });
-    const int slot = iolet_fixup<S>(D, s, g);
-    const float4 m = collide_s<S>(g, D.omega);
-    typename St<S>::T *wb = opaque(buf);
-    wb[s] = Tr::template st<0>(g[0]);
-    const int32_t *nb2 = opaque(D.nbr);  // each store's entry reread right before it (cache hit)
-    unroll<1, 19>([&](auto ic) {
-        constexpr int I = decltype(ic)::v;
-        wb[(int64_t)I * np + __ldg(nb2 + (int64_t)(OPP(I) - 1) * np + s)] = Tr::template st<I>(g[I]);
-    });
-    if (slot >= 0) D.bnd[slot] = m;
-}
-
-// ==== async-staged variant (V = 1) ==========================================
-// The 19 gathers of every site a thread owns are issued as cp.async copies into
-// a shared-memory stage [SPT][19][blockDim] (4-byte words) before one wait, so
-// the loads in flight do not hold registers.  16-bit elements are fetched as
-// the aligned 32-bit word that contains them; `sel` remembers which half.
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-}
-
-template <int S> struct Word;
-template <> struct Word<kF32> {
-    static __device__ __forceinline__ const void *src(const float *p, uint32_t &sel, int) {
-        return p;
-    }
-    template <int I> static __device__ __forceinline__ float get(uint32_t w, uint32_t) {
-        return __uint_as_float(w);
-    }
-};
-template <int S16> struct Word16 {
-    using T = typename St<S16>::T;
-    static __device__ __forceinline__ const void *src(const T *p, uint32_t &sel, int I) {
-        const uintptr_t a = (uintptr_t)p;
-        sel |= (uint32_t)((a >> 1) & 1u) << I;
-        return (const void *)(a & ~(uintptr_t)3);
-    }
-    template <int I> static __device__ __forceinline__ float get(uint32_t w, uint32_t sel) {
-        const unsigned short h = (unsigned short)(((sel >> I) & 1u) ? (w >> 16) : (w & 0xffffu));
-        if constexpr (S16 == kF16) return St<kF16>::template ld<I>(__ushort_as_half(h));
-        else return St<kBF16>::template ld<I>(__ushort_as_bfloat16(h));
-    }
-};
-template <> struct Word<kF16> : Word16<kF16> {};
-template <> struct Word<kBF16> : Word16<kBF16> {};
-
-// Issue the gathers of site s (virtual indices: one formula for every link).
-// A/B pulls slot I from x - c_I; AA odd pulls the swapped slot OPP(I).
-template <int S, bool AA>
-__device__ __forceinline__ uint32_t issue_gathers(const DomDev &D, const typename St<S>::T *src,
-                                                  int64_t s, uint32_t stage, uint32_t rstride) {
-    const int64_t np = D.np;
-    uint32_t sel = 0;
-    int32_t nb[18];
-#pragma unroll
-    for (int i = 0; i < 18; ++i) nb[i] = __ldg(D.nbr + (int64_t)i * np + s);
-    cp_async4(stage, Word<S>::src(src + s, sel, 0));
-    unroll<1, 19>([&](auto ic) {
-        constexpr int I = decltype(ic)::v;
-        const typename St<S>::T *p = src + ((int64_t)(AA ? OPP(I) : I) * np + nb[I - 1]);
-        cp_async4(stage + I * rstride, Word<S>::src(p, sel, I));
-    });
-    return sel;
-}
-
-template <int S>
-__device__ __forceinline__ void read_staged(const uint32_t *st, uint32_t rwords, uint32_t sel,
-                                            float g[19]) {
-    unroll<0, 19>([&](auto ic) {
-        constexpr int I = decltype(ic)::v;
-        g[I] = Word<S>::template get<I>(st[I * rwords], sel);
-    });
-}
-
-template <int S, int SPT>
-__device__ __forceinline__ void tile_ab_async(const DomDev &D, const TileDev &tl, bool odd,
-                                              uint32_t *stage_base) {
-    using T = typename St<S>::T;
-    const T *src = (const T *)D.f[odd ? 0 : 1];  // F_{t-1} sits in f[(t-1) & 1]
-    T *dst = (T *)D.f[odd ? 1 : 0];
-    const uint32_t B = blockDim.x;
-    uint32_t sel[SPT];
-#pragma unroll
-    for (int j = 0; j < SPT; ++j) {
-        const int r = j * B + threadIdx.x;
-        sel[j] = r < tl.count ? issue_gathers<S, false>(D, src, tl.start + r,
-                                                        smem_addr(stage_base + (j * 19) * B + threadIdx.x), 4 * B)
-                              : 0u;
-    }
-    cp_async_wait_all();
-#pragma unroll
-    for (int j = 0; j < SPT; ++j) {
-        const int r = j * B + threadIdx.x;
-        if (r >= tl.count) continue;
-        const int64_t s = tl.start + r;
-        float g[19];
-        read_staged<S>(stage_base + (j * 19) * B + threadIdx.x, B, sel[j], g);
-        const int slot = iolet_fixup<S>(D, s, g);
-        const float4 m = collide_s<S>(g, D.omega);
-        T *wb = opaque(dst + s);
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            wb[(int64_t)I * D.np] = St<S>::template st<I>(g[I]);
-        });
-        if (slot >= 0) D.bnd[slot] = m;
-    }
-}
-
-template <int S, int SPT>
-__device__ __forceinline__ void tile_aa_odd_async(const DomDev &D, const TileDev &tl,
-                                                  uint32_t *stage_base) {
-    using T = typename St<S>::T;
-    T *buf = (T *)D.f[0];
-    const uint32_t B = blockDim.x;
-    uint32_t sel[SPT];
-#pragma unroll
-    for (int j = 0; j < SPT; ++j) {
-        const int r = j * B + threadIdx.x;
-        sel[j] = r < tl.count ? issue_gathers<S, true>(D, buf, tl.start + r,
-                                                       smem_addr(stage_base + (j * 19) * B + threadIdx.x), 4 * B)
-                              : 0u;
-    }
-    cp_async_wait_all();
-#pragma unroll
-    for (int j = 0; j < SPT; ++j) {
-        const int r = j * B + threadIdx.x;
-        if (r >= tl.count) continue;
-        const int64_t s = tl.start + r;
-        float g[19];
-        read_staged<S>(stage_base + (j * 19) * B + threadIdx.x, B, sel[j], g);
-        const int slot = iolet_fixup<S>(D, s, g);
-        const float4 m = collide_s<S>(g, D.omega);
-        const int32_t *nb2 = opaque(D.nbr);  // fresh (L1-resident) reads for the scatter
-        T *wb = opaque(buf);
-        const int64_t np = D.np;
-        wb[s] = St<S>::template st<0>(g[0]);
-        unroll<1, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            const int32_t tg = __ldg(nb2 + (int64_t)(OPP(I) - 1) * np + s);  // site at x + c_I
-            wb[(int64_t)I * np + tg] = St<S>::template st<I>(g[I]);
-        });
-        if (slot >= 0) D.bnd[slot] = m;
-    }
-}
-
-// ==== staged-scatter AA odd step (V = 4, one site per thread) ===============
-// The odd step stores the value of direction I at x + c_I.  Most of those
-// targets lie in the same tile: their values are parked in the gather stage
-// (free once every thread has read its gathers) at the target's position and
-// then written row by row with coalesced stores.  A target outside the tile
-// gets its value directly; a non-fluid target parks the raw value at the own
-// site's slot OPP(I).  Position p's row-I value comes from the pull source of
-// direction I at p (its own neighbour-table entry I), or from p itself when
-// that entry is virtual; entry I is also the target entry of p's own
-// direction OPP(I), so the scatter pass records in one bit per row whether the
-// tile holds position p's value.  Each location is read and written by one
-// site only (the AA property), so the deferred stores race with no other tile.
-template <int S>
-__device__ __forceinline__ void tile_aa_odd_staged(const DomDev &D, const TileDev &tl, uint32_t *stage) {
-    using T = typename St<S>::T;
-    T *buf = (T *)D.f[0];
-    const uint32_t B = blockDim.x;
-    const int r = threadIdx.x;
-    const bool live = r < tl.count;
-    const int64_t s = tl.start + r;
-    const int64_t np = D.np;
-    const uint32_t sel = live ? issue_gathers<S, true>(D, buf, s, smem_addr(stage + r), 4 * B) : 0u;
-    cp_async_wait_all();
-    float g[19];
-    int slot = -1;
-    float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (live) {
-        read_staged<S>(stage + r, B, sel, g);
-        slot = iolet_fixup<S>(D, s, g);
-        m = collide_s<S>(g, D.omega);
-    }
-    __syncthreads();  // every gather has been read: the stage now takes outputs
-    uint32_t held = 0;  // bit J: the tile holds this position's row-J value
-    if (live) {
-        const int32_t *nb2 = opaque(D.nbr);
-        T *wb = opaque(buf);
-        wb[s] = St<S>::template st<0>(g[0]);
-        unroll<1, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            const int32_t tg = __ldg(nb2 + (int64_t)(OPP(I) - 1) * np + s);  // site at x + c_I
-            const int64_t rel = (int64_t)tg - tl.start;
-            if ((uint64_t)rel < (uint64_t)tl.count) {
-                stage[I * B + (uint32_t)rel] = __float_as_uint(g[I]);
-                held |= 1u << OPP(I);
-            } else if (tg < 0 || tg >= np) {
-                stage[OPP(I) * B + r] = __float_as_uint(g[I]);
-                held |= 1u << OPP(I);
-            } else {
-                wb[(int64_t)I * np + tg] = St<S>::template st<I>(g[I]);
-            }
-        });
-        if (slot >= 0) D.bnd[slot] = m;
-    }
-    __syncthreads();
-    if (live) {
-        T *wb = opaque(buf);
-        unroll<1, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            if ((held >> I) & 1u)
-                wb[(int64_t)I * np + s] = St<S>::template st<I>(__uint_as_float(stage[I * B + r]));
-        });
-    }
-}
-
-// AA even step on pairs of adjacent sites (2 per thread): vector loads/stores.
+// ---- pairs of adjacent sites: vector loads and stores, packed arithmetic ----
 template <int S> struct Pair;
 template <> struct Pair<kF32> {
     template <int I> static __device__ __forceinline__ void ld(const float *p, float &a, float &b) {
@@ -804,10 +540,11 @@ __device__ __forceinline__ void put_moments(const DomDev &D, int slot_a, int slo
     if (slot_b >= 0) D.bnd[slot_b] = mom_hi(m);
 }
 
-// ---- A/B pull on a pair of adjacent sites (variant 5, 16-bit storage) ----
+// ---- A/B pull on a pair of adjacent sites (18-row table, 16-bit storage) ----
 // Sites s and s+1 (s even) share one 8-byte load per neighbour-table row, one
 // 4-byte load of the rest values and one 4-byte store per direction: fewer
-// memory instructions per site for a kernel that runs near its issue limit.
+// memory instructions per site for a kernel that runs near its issue limit
+// (~10M-site tree in rows: 221 us against 252 for one site per thread).
 template <int S>
 __device__ __forceinline__ void site_ab_pair(const DomDev &D, const typename St<S>::T *__restrict__ src,
                                              typename St<S>::T *__restrict__ dst, int64_t s) {
@@ -828,38 +565,6 @@ __device__ __forceinline__ void site_ab_pair(const DomDev &D, const typename St<
     unroll<0, 19>([&](auto ic) {
         constexpr int I = decltype(ic)::v;
         st_pair<S, I>(wb + (int64_t)I * np, g[I]);
-    });
-    put_moments(D, slot_a, slot_b, m);
-}
-
-// ---- AA on a pair of adjacent sites (variant 6 / 7: 7 adds L2 prefetch hints) ----
-// Sites s and s+1 (s even) share one 8-byte load per neighbour-table row, both for
-// the gathers and for the re-read that addresses the scatter, and one load and one
-// store of their two rest values; the 18 gathers and 18 scattered stores stay per
-// site.  The odd step reads slot OPP(I) at x - c_I and writes slot I at x + c_I.
-template <int S, bool HINT>
-__device__ __forceinline__ void site_aa_odd_pair(const DomDev &D, typename St<S>::T *buf, int64_t s) {
-    using Tr = St<S>;
-    const int64_t np = D.np;
-    F2 g[19];
-    g[0] = ld_pair<S, 0>(buf + s);
-    unroll<1, 19>([&](auto ic) {
-        constexpr int I = decltype(ic)::v;
-        const int2 nb = __ldg(reinterpret_cast<const int2 *>(D.nbr + (int64_t)(I - 1) * np + s));
-        g[I] = pk2(Tr::template ld<I>(load_rw<HINT>(buf + ((int64_t)OPP(I) * np + nb.x))),
-                   Tr::template ld<I>(load_rw<HINT>(buf + ((int64_t)OPP(I) * np + nb.y))));
-    });
-    int slot_a, slot_b;
-    iolet_fixup2<S>(D, s, s + 1, g, slot_a, slot_b);
-    const MomT<F2> m = collide_v<Tr::kScaled>(g, D.omega, D.neg_zero2);
-    typename St<S>::T *wb = opaque(buf);
-    const int32_t *nb2 = opaque(D.nbr);  // reread (L1 hits) instead of keeping 36 entries live
-    st_pair<S, 0>(wb + s, g[0]);
-    unroll<1, 19>([&](auto ic) {
-        constexpr int I = decltype(ic)::v;
-        const int2 tg = __ldg(reinterpret_cast<const int2 *>(nb2 + (int64_t)(OPP(I) - 1) * np + s));
-        wb[(int64_t)I * np + tg.x] = Tr::template st<I>(lo2(g[I]));
-        wb[(int64_t)I * np + tg.y] = Tr::template st<I>(hi2(g[I]));
     });
     put_moments(D, slot_a, slot_b, m);
 }
@@ -895,19 +600,23 @@ __device__ __forceinline__ void tile_aa_even_pairs(const DomDev &D, const TileDe
     }
 }
 
-// ==== run-encoded form (variants 8..14) ========================================
-// What bounds it: for 16-bit storage instruction issue (68 % of the slots; 438 instructions
+// ==== one site per thread: the A/B step and the AA odd step ====================
+// With the run encoding -- what bounds it: for 16-bit storage instruction issue (68 % of the slots; 438 instructions
 // per site and A/B step, 518 before the links were decoded as below), for FP32 HBM (A/B) and
 // the misaligned scatter (AA odd).  40 registers, so 48 warps per SM hide the chain word ->
 // run row -> gathers.  ~10M-site tree, stream-collide alone, before -> now: FP32 A/B 243 ->
-// 241 us, FP16 A/B 192 -> 181, FP32 AA odd 303 -> 272, FP16 AA odd 236 -> 198 (even 123).
+// 236 us, FP16 A/B 192 -> 178, FP32 AA odd 303 -> 268, FP16 AA odd 236 -> 197 (even 119).
 // Tried and slower: two sites per thread with packed arithmetic (350 instructions per site,
 // but 64-90 registers: 188-230 us FP16 A/B); lists of all-fluid pairs and single sites (250
 // instructions per site, but the lists' stores leave sectors half written: FP32 A/B 296 us);
 // an L2 prefetch of the rows 64K..1M sites ahead (no change to 20 % slower).
-template <int S, int SCHEME> __device__ __forceinline__ float run_ld(const typename St<S>::T *p) {
-    if constexpr (SCHEME == kAA) return St<S>::template ld<0>(load_rw<true>(p));
-    else return St<S>::template ld<0>(load_ro<true>(p));
+// With the 18-row table it is bound by the table's 72 bytes and the scattered sectors of
+// Morton order (~10M-site tree, Morton / rows): FP32 A/B 330 / 320 us (475 before the 32-bit
+// multiply-add addresses), FP16 AA odd 343 / 260 and FP32 AA odd 429 / 340, against 391 / 346
+// and 471 / 428 for gathers staged by cp.async and 393 / 272 and 483 / 354 for adjacent pairs.
+template <int S, int SCHEME, bool HINT> __device__ __forceinline__ float link_ld(const typename St<S>::T *p) {
+    if constexpr (SCHEME == kAA) return St<S>::template ld<0>(load_rw<HINT>(p));
+    else return St<S>::template ld<0>(load_ro<HINT>(p));
 }
 struct RunSite {
     uint32_t w;
@@ -919,29 +628,54 @@ __device__ __forceinline__ RunSite run_site(const DomDev &D, int64_t s) {
     r.row = D.rdelta + (int64_t)(__ldg(D.run0 + (s >> 10)) + (int32_t)((r.w >> 18) & 1023u)) * kRunStride;
     return r;
 }
-// A/B step or AA odd step of one site whose word and run row are at hand.  The AA scatter
-// goes to the places the gather read (direction I where its opposite was read); their 18
-// offsets wait in shared memory, one bank per thread, instead of being decoded again.
-template <int S, int SCHEME>
-__device__ __forceinline__ void site_run(const DomDev &D, const typename St<S>::T *src, typename St<S>::T *dst,
-                                         int64_t s, const RunSite &r, int32_t *stash) {
+// The links of a site as offsets from the own site in the first row of the link's opposite
+// pair: each(f) calls f(IC<I>, offset) for I = 1..18.
+template <int SCHEME> struct RunOffsets {
+    RunSite r;
+    int32_t np;
+    template <typename F> __device__ __forceinline__ void each(F &&f) const {
+        unroll<0, 5>([&](auto kc) {
+            run_links4<decltype(kc)::v>(r.row, [&](auto ic, int32_t d) {
+                f(ic, run_offset<SCHEME, decltype(ic)::v>(r.w, d, np));
+            });
+        });
+    }
+    __device__ __forceinline__ bool next_to_iolet(const DomDev &, int64_t) const { return r.w >> 31; }
+};
+template <int SCHEME, bool HINT> struct TableOffsets {
+    const int32_t *p;  // entry 1 of the site
+    int32_t s, np;
+    template <typename F> __device__ __forceinline__ void each(F &&f) const {
+        unroll<1, 19>([&](auto ic) {
+            constexpr int I = decltype(ic)::v;
+            constexpr bool second = SCHEME == kAB ? (I & 1) == 0 : (I & 1) != 0;  // the row gathered from
+            f(ic, load_nbr<HINT>(p + (int64_t)(I - 1) * np) - s + (second ? np : 0));
+        });
+    }
+    __device__ __forceinline__ bool next_to_iolet(const DomDev &D, int64_t at) const {
+        uint32_t word;
+        return site_flag(D, at, word);
+    }
+};
+// A/B step or AA odd step of one site.  The AA scatter goes to the places the gather read
+// (direction I where its opposite was read); their 18 offsets wait in shared memory, one bank
+// per thread (`stash`: this thread's), instead of being decoded again.
+template <int S, int SCHEME, bool HINT, typename L>
+__device__ __forceinline__ void site_links(const DomDev &D, const typename St<S>::T *src, typename St<S>::T *dst,
+                                           int64_t s, const L &links, int32_t *stash) {
     using Tr = St<S>;
     using T = typename Tr::T;
-    const int32_t np = (int32_t)D.np;
     const uint32_t npb = (uint32_t)D.np * sizeof(T);
     const T *p = src + s;
     float g[19];
-    g[0] = run_ld<S, SCHEME>(p);
-    unroll<0, 5>([&](auto kc) {
-        run_links4<decltype(kc)::v>(r.row, [&](auto ic, int32_t d) {
-            constexpr int I = decltype(ic)::v;
-            const int32_t off = run_offset<SCHEME, I>(r.w, d, np);
-            g[I] = run_ld<S, SCHEME>(pair_row<I>(p, npb) + off);
-            if constexpr (SCHEME == kAA) stash[(I - 1) * blockDim.x] = off;
-        });
+    g[0] = link_ld<S, SCHEME, HINT>(p);
+    links.each([&](auto ic, int32_t off) {
+        constexpr int I = decltype(ic)::v;
+        g[I] = link_ld<S, SCHEME, HINT>(pair_row<I>(p, npb) + off);
+        if constexpr (SCHEME == kAA) stash[(I - 1) * blockDim.x] = off;
     });
     int slot = -1;
-    if (r.w >> 31) {  // a link into an iolet opening
+    if (links.next_to_iolet(D, s)) {
         wait_for_iolet_update();
         slot = site_slot(D, s, __ldg(D.iomask + (s >> 5)));
         apply_iolet_links<S>(D, D.bcv, slot, io_word(D, slot), g);
@@ -985,171 +719,49 @@ __device__ __forceinline__ void tile_runs(const DomDev &D, const TileDev &tl, co
 #pragma unroll
     for (int j = 0; j < SPT; ++j) {
         const int q = j * blockDim.x + threadIdx.x;
-        if (q < tl.count) site_run<S, SCHEME>(D, src, dst, tl.start + q, r[j], stash + threadIdx.x);
-    }
-}
-
-// ==== TMA bulk-copy AA even step (V = 2) ======================================
-// One thread moves the tile's 19 rows (contiguous segments of the SoA arrays)
-// into shared memory with cp.async.bulk, completion tracked by an mbarrier;
-// every thread collides its sites from shared memory, writes the swapped
-// result back into the same column, and one thread stores the 19 rows with
-// bulk copies.  The wait is bounded: on timeout the context error word is set.
-constexpr uint32_t kWaitLimit = 1u << 22;
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity) {
-    for (uint32_t it = 0; it < kWaitLimit; ++it)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-__device__ __forceinline__ void bulk_g2s(void *sdst, const void *gsrc, uint32_t bytes, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_addr(sdst)),
-        "l"(gsrc), "r"(bytes), "r"(smem_addr(bar))
-        : "memory");
-}
-__device__ __forceinline__ void bulk_s2g(void *gdst, const void *ssrc, uint32_t bytes) {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst), "r"(smem_addr(ssrc)),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_commit_wait_read() {
-    asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group.read 0;\n" ::: "memory");
-}
-
-template <int S>
-__device__ __forceinline__ void tile_aa_even_tma(const DomDev &D, const TileDev &tl, uint32_t cap,
-                                                 unsigned char *smem) {
-    using T = typename St<S>::T;
-    constexpr uint32_t E = sizeof(T);
-    T *buf = (T *)D.f[0];
-    const int64_t np = D.np;
-    uint64_t *bar = (uint64_t *)smem;
-    T *rows = (T *)(smem + 16);
-    const uint32_t bytes = ((uint32_t)tl.count * E + 15u) & ~15u;  // padding keeps it inside the row
-    if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        mbar_expect_tx(bar, 19u * bytes);
-        for (int I = 0; I < 19; ++I) bulk_g2s(rows + (size_t)I * cap, buf + (int64_t)I * np + tl.start, bytes, bar);
-    }
-    const bool ok = __syncthreads_and(mbar_wait_bounded(bar, 0));
-    if (!ok) {  // never expected: report, let the copies land, leave the tile untouched
-        if (threadIdx.x == 0) atomicExch(D.err, 1);
-        mbar_wait_bounded(bar, 0);
-        return;
-    }
-    for (int r = threadIdx.x; r < tl.count; r += blockDim.x) {
-        const int64_t s = tl.start + r;
-        float g[19];
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            g[I] = St<S>::template ld<I>(rows[(size_t)I * cap + r]);
-        });
-        const int slot = iolet_fixup<S>(D, s, g);
-        const float4 m = collide_s<S>(g, D.omega);
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            rows[(size_t)OPP(I) * cap + r] = St<S>::template st<I>(g[I]);
-        });
-        if (slot >= 0) D.bnd[slot] = m;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int I = 0; I < 19; ++I) bulk_s2g(buf + (int64_t)I * np + tl.start, rows + (size_t)I * cap, bytes);
-        bulk_commit_wait_read();
+        if (q < tl.count)
+            site_links<S, SCHEME, true>(D, src, dst, tl.start + q, RunOffsets<SCHEME>{r[j], (int32_t)D.np}, stash);
     }
 }
 
 // PAR is the parity of the step this launch executes: 0 = even, 1 = odd (the
 // AA step kind), 2 = read from the domain's step counter per block (A/B, and AA
-// batches whose domains are at different parities).
-// One tile of one domain, after the prologue has located it.  Variants 8..14 are one kernel
-// (V = 8), which reads the run-encoded neighbour table.  The host launches it only on domains
-// that have one (the others get a table form); a domain without one here is reported through
-// the error word (code 2) and left untouched.
-constexpr bool hinted(int v) { return v == 3 || v == 7; }
-template <int S, int SCHEME, int SPT, int PAR, int V>
-__device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileDev &tl, bool odd,
-                                                    uint32_t *stage) {
+// batches whose domains are at different parities).  RUNS: the domain has a run
+// encoding (the host launches the form only on such domains; a domain without one here is
+// reported through the error word, code 2, and left untouched).
+// One tile of one domain, after the prologue has located it.
+template <int S, int SCHEME, int PAR, bool RUNS>
+__device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileDev &tl, bool odd, int32_t *stash) {
     using T = typename St<S>::T;
-    constexpr bool HINT = hinted(V);
-    if constexpr (V == 8) {
-        if (D.lword == nullptr) {
-            if (threadIdx.x == 0) atomicExch(D.err, 2);
-            return;
-        }
-        if (SCHEME == kAB || PAR == 1 || (PAR == 2 && odd))
-            tile_runs<S, SCHEME, SPT>(D, tl, (const T *)D.f[SCHEME == kAA || odd ? 0 : 1],
-                                            (T *)D.f[SCHEME == kAA || !odd ? 0 : 1], (int32_t *)stage);
-        else tile_aa_even_pairs<S>(D, tl);
-    } else if constexpr (V == 1 || V == 2 || V == 4) {
-        if constexpr (SCHEME == kAB) {
-            tile_ab_async<S, SPT>(D, tl, odd, stage);
-        } else {
-            if (odd) {
-                if constexpr (V == 4) tile_aa_odd_staged<S>(D, tl, stage);
-                else tile_aa_odd_async<S, SPT>(D, tl, stage);
-            } else if constexpr (V == 2) {
-                tile_aa_even_tma<S>(D, tl, (uint32_t)(SPT * blockDim.x), (unsigned char *)stage);
-            } else {
-                tile_aa_even_pairs<S>(D, tl);
-            }
-        }
-    } else if constexpr (V == 6 || V == 7) {
-        // AA on adjacent pairs: each thread takes sites 2t and 2t+1 of the tile (SPT = 2)
-        static_assert(SCHEME == kAA && SPT == 2, "variants 6 and 7 are the AA pair forms");
-        T *buf = (T *)D.f[0];
-        const int r = 2 * threadIdx.x;
-        const int64_t s = tl.start + r;  // even: tiles start at multiples of 2 * blockDim
-        if (r + 1 < tl.count) {
-            if (odd) site_aa_odd_pair<S, HINT>(D, buf, s);
-            else site_aa_even_pair<S>(D, buf, s);
-        } else if (r < tl.count) {  // ragged tail: one site
-            if (odd) site_aa_odd<S, HINT>(D, buf, s);
-            else site_aa_even<S, HINT>(D, buf, s);
-        }
-    } else if constexpr (V == 5) {
-        // A/B on adjacent pairs: each thread takes sites 2t and 2t+1 of the tile (SPT = 2)
-        static_assert(SCHEME == kAB && SPT == 2, "variant 5 is the A/B pair form");
-        const int r = 2 * threadIdx.x;
-        const int64_t s = tl.start + r;  // even: tiles start at multiples of 2 * blockDim
-        const T *src = (const T *)D.f[odd ? 0 : 1];
-        T *dst = (T *)D.f[odd ? 1 : 0];
-        if (r + 1 < tl.count) site_ab_pair<S>(D, src, dst, s);
-        else if (r < tl.count) site_ab<S>(D, src, dst, s);  // ragged tail: one site
+    constexpr int SPT = sc_spt(S, SCHEME, PAR, RUNS);
+    if (RUNS && D.lword == nullptr) {
+        if (threadIdx.x == 0) atomicExch(D.err, 2);
+        return;
+    }
+    if (SCHEME == kAA && (PAR == 0 || (PAR == 2 && !odd))) {
+        tile_aa_even_pairs<S>(D, tl);
+        return;
+    }
+    const T *src = (const T *)D.f[SCHEME == kAA || odd ? 0 : 1];  // A/B: F_{t-1} sits in f[(t-1) & 1]
+    T *dst = (T *)D.f[SCHEME == kAA || !odd ? 0 : 1];
+    if constexpr (RUNS) {
+        tile_runs<S, SCHEME, SPT>(D, tl, src, dst, stash);
     } else {
+        // FP32 AA without the 256-byte hints: 429 us against 446 (Morton), 340 against 346 (rows)
+        constexpr bool HINT = !(SCHEME == kAA && S == kF32);
+        auto one_site = [&](int64_t s) {
+            site_links<S, SCHEME, HINT>(D, src, dst, s,
+                                        TableOffsets<SCHEME, HINT>{D.nbr + s, (int32_t)s, (int32_t)D.np}, stash);
+        };
+        if constexpr (SCHEME == kAB && S != kF32) {
+            const int r = 2 * threadIdx.x;  // even sites: tiles start at multiples of kTile
+            if (r + 1 < tl.count) site_ab_pair<S>(D, src, dst, tl.start + r);
+            else if (r < tl.count) one_site(tl.start + r);
+        } else {
 #pragma unroll
-        for (int j = 0; j < SPT; ++j) {
-            const int r = j * blockDim.x + threadIdx.x;
-            const int64_t s = tl.start + r;
-            if (r >= tl.count) continue;
-            if constexpr (SCHEME == kAB) {
-                site_ab<S, HINT>(D, (const T *)D.f[odd ? 0 : 1], (T *)D.f[odd ? 1 : 0], s);
-            } else {
-                if (odd) site_aa_odd<S, HINT>(D, (T *)D.f[0], s);
-                else site_aa_even<S, HINT>(D, (T *)D.f[0], s);
+            for (int j = 0; j < SPT; ++j) {
+                const int r = j * blockDim.x + threadIdx.x;
+                if (r < tl.count) one_site(tl.start + r);
             }
         }
     }
@@ -1158,15 +770,15 @@ __device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileD
 // Many domains per launch: each block finds its tile in the tile table; the
 // first threads copy the tile's domain descriptor into shared memory, one
 // 8-byte word each, while thread 0 reads the domain's step counter.
-template <int S, int SCHEME, int SPT, int PAR, int V>
+template <int S, int SCHEME, int PAR, bool RUNS>
 __global__ void __launch_bounds__(512) k_stream_collide(const DomDev *__restrict__ doms,
-                                                        const TileDev *__restrict__ tiles,
-                                                        const int64_t *__restrict__ steps, int off) {
+                                                          const TileDev *__restrict__ tiles,
+                                                          const int64_t *__restrict__ steps, int off) {
     static_assert(sizeof(DomDev) % 8 == 0, "descriptor copied in 8-byte words");
     constexpr int kWords = (int)(sizeof(DomDev) / 8);
     __shared__ DomDev D;
     __shared__ int64_t t_now;
-    extern __shared__ __align__(128) uint32_t stage[];
+    extern __shared__ __align__(128) int32_t stash[];
     const TileDev tl = tiles[blockIdx.x];
     if (threadIdx.x < kWords)
         reinterpret_cast<uint64_t *>(&D)[threadIdx.x] =
@@ -1177,21 +789,20 @@ __global__ void __launch_bounds__(512) k_stream_collide(const DomDev *__restrict
         if (threadIdx.x == 0) t_now = __ldg(steps + tl.dom) + off + 1;
     __syncthreads();
     const bool odd = PAR == 2 ? (t_now & 1) != 0 : PAR == 1;
-    stream_collide_tile<S, SCHEME, SPT, PAR, V>(D, tl, odd, stage);
+    stream_collide_tile<S, SCHEME, PAR, RUNS>(D, tl, odd, stash + threadIdx.x);
 }
 
 // One domain per launch: the descriptor is a kernel parameter (constant bank)
-// and block b takes units [b*T, b*T + T) of the n (sites, or tasks: tile_units), so no
+// and block b takes sites [b*T, b*T + T) with T = sites per thread * blockDim, so no
 // block waits on a table load or a barrier before its first neighbour-table load.
-template <int S, int SCHEME, int SPT, int PAR, int V>
-__global__ void __launch_bounds__(512) k_stream_collide_one(const __grid_constant__ DomDev D, int64_t n,
-                                                            int off) {
+template <int S, int SCHEME, int PAR, bool RUNS>
+__global__ void __launch_bounds__(512) k_stream_collide_one(const __grid_constant__ DomDev D, int64_t n, int off) {
     // a launch chained after this one (the next domain of a per-domain launch
     // sequence) may be scheduled once every block here has started; kernels launched
     // without programmatic serialisation ignore the trigger
     asm volatile("griddepcontrol.launch_dependents;");
-    extern __shared__ __align__(128) uint32_t stage[];
-    const int64_t ts = (int64_t)SPT * blockDim.x;
+    extern __shared__ __align__(128) int32_t stash[];
+    const int64_t ts = (int64_t)sc_spt(S, SCHEME, PAR, RUNS) * blockDim.x;
     TileDev tl;
     tl.dom = 0;
     tl.start = (int64_t)blockIdx.x * ts;
@@ -1199,94 +810,25 @@ __global__ void __launch_bounds__(512) k_stream_collide_one(const __grid_constan
     bool odd;
     if constexpr (PAR == 2) odd = ((__ldg(D.step) + off + 1) & 1) != 0;
     else odd = PAR == 1;
-    stream_collide_tile<S, SCHEME, SPT, PAR, V>(D, tl, odd, stage);
+    stream_collide_tile<S, SCHEME, PAR, RUNS>(D, tl, odd, stash + threadIdx.x);
 }
 
-
-template <int S, int SCHEME, int PAR, int V, int SPT>
-cudaError_t launch_sc_one(const CollideCfg &cfg, const DomDev *doms, const TileDev *tiles,
-                          int64_t n_tiles, int off, const OneDomain &one, cudaStream_t st) {
-    // V1/V4: cp.async stage of 4-byte words (V4 reuses it for the odd step's outputs);
-    // V2 also holds the even step's 19 rows + mbarrier
-    size_t smem = (V == 1 || V == 2 || V == 4) ? (size_t)SPT * 19 * cfg.block * 4 : 0;
-    if (V == 2) smem += 16;
-    if (V == 8 && SCHEME == kAA && PAR != 0) smem = (size_t)18 * 4 * cfg.block;  // odd step's offsets
+template <int S, int SCHEME, int PAR, bool RUNS>
+cudaError_t launch_sc(const CollideCfg &cfg, const DomDev *doms, const TileDev *tiles, int64_t n_tiles, int off,
+                      const OneDomain &one, cudaStream_t st) {
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)n_tiles);
     lc.blockDim = dim3((unsigned)cfg.block);
-    lc.dynamicSmemBytes = smem;
+    // the AA odd step's 18 offsets per thread
+    lc.dynamicSmemBytes = SCHEME == kAA && PAR != 0 ? (size_t)18 * 4 * cfg.block : 0;
     lc.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = one.overlap_previous ? 1 : 0;  // start while the previous iolet update runs
-    if (one.d) {
-        auto k = k_stream_collide_one<S, SCHEME, SPT, PAR, V>;
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        return cudaLaunchKernelEx(&lc, k, *one.d, one.n, off);
-    }
-    auto k = k_stream_collide<S, SCHEME, SPT, PAR, V>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaLaunchKernelEx(&lc, k, doms, tiles, one.steps, off);
-}
-
-template <int S, int SCHEME, int PAR>
-cudaError_t launch_sc_spt(const CollideCfg &cfg, const DomDev *doms, const TileDev *tiles,
-                          int64_t n_tiles, int off, const OneDomain &one, cudaStream_t st) {
-    if (cfg.variant == 1) {
-        switch (cfg.spt) {
-            case 1: return launch_sc_one<S, SCHEME, PAR, 1, 1>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 2: return launch_sc_one<S, SCHEME, PAR, 1, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (cfg.variant == 3) {
-        switch (cfg.spt) {
-            case 1: return launch_sc_one<S, SCHEME, PAR, 3, 1>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 2: return launch_sc_one<S, SCHEME, PAR, 3, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 4: return launch_sc_one<S, SCHEME, PAR, 3, 4>(cfg, doms, tiles, n_tiles, off, one, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (cfg.variant == 4) {
-        if constexpr (SCHEME == kAB) return cudaErrorInvalidValue;
-        else if (cfg.spt != 1) return cudaErrorInvalidValue;
-        else return launch_sc_one<S, SCHEME, PAR, 4, 1>(cfg, doms, tiles, n_tiles, off, one, st);
-    }
-    if (cfg.variant == 5) {
-        if constexpr (SCHEME != kAB || S == kF32) return cudaErrorInvalidValue;
-        else if (cfg.spt != 2) return cudaErrorInvalidValue;
-        else return launch_sc_one<S, SCHEME, PAR, 5, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-    }
-    if (cfg.variant == 6 || cfg.variant == 7) {
-        if constexpr (SCHEME != kAA) return cudaErrorInvalidValue;
-        else if (cfg.spt != 2) return cudaErrorInvalidValue;
-        else if (cfg.variant == 6) return launch_sc_one<S, SCHEME, PAR, 6, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-        else return launch_sc_one<S, SCHEME, PAR, 7, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-    }
-    if (cfg.variant >= 8)
-        return launch_sc_one<S, SCHEME, PAR, 8, run_spt(S, SCHEME, PAR)>(cfg, doms, tiles, n_tiles, off, one, st);
-    if (cfg.variant == 2) {
-        if (SCHEME == kAB) return cudaErrorInvalidValue;
-        switch (cfg.spt) {
-            case 1: return launch_sc_one<S, SCHEME, PAR, 2, 1>(cfg, doms, tiles, n_tiles, off, one, st);
-            case 2: return launch_sc_one<S, SCHEME, PAR, 2, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    switch (cfg.spt) {
-        case 1: return launch_sc_one<S, SCHEME, PAR, 0, 1>(cfg, doms, tiles, n_tiles, off, one, st);
-        case 2: return launch_sc_one<S, SCHEME, PAR, 0, 2>(cfg, doms, tiles, n_tiles, off, one, st);
-        case 4: return launch_sc_one<S, SCHEME, PAR, 0, 4>(cfg, doms, tiles, n_tiles, off, one, st);
-        default: return cudaErrorInvalidValue;
-    }
+    if (one.d) return cudaLaunchKernelEx(&lc, k_stream_collide_one<S, SCHEME, PAR, RUNS>, *one.d, one.n, off);
+    return cudaLaunchKernelEx(&lc, k_stream_collide<S, SCHEME, PAR, RUNS>, doms, tiles, one.steps, off);
 }
 
 }  // namespace

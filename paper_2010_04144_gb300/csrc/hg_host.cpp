@@ -712,7 +712,7 @@ const DomDev *domdev_ptr(hg_domain *d) {
 
 size_t elem_bytes(int storage) { return storage == HG_STORE_F32 ? 4 : 2; }
 
-// Kernel variants and the launch shapes each supports (see hg_ctx_params).
+// Kernel variants and the launch shapes accepted with each (see hg_ctx_params).
 bool variant_ok(int storage, int scheme, int spt, int variant) {
     switch (variant) {
         case 0: case 3: return true;
@@ -721,7 +721,7 @@ bool variant_ok(int storage, int scheme, int spt, int variant) {
         case 4: return spt == 1 && scheme == HG_SCHEME_AA;
         case 5: return spt == 2 && scheme == HG_SCHEME_AB && storage != HG_STORE_F32;
         case 6: case 7: return spt == 2 && scheme == HG_SCHEME_AA;
-        case 8: return true;  // 8..11: variants 3, 5, 6, 7 reading the run-encoded table
+        case 8: return true;
         case 9: return spt == 2 && scheme == HG_SCHEME_AB && storage != HG_STORE_F32;
         case 10: case 11: return spt == 2 && scheme == HG_SCHEME_AA;
         case 12: return spt != 4 && scheme == HG_SCHEME_AA;
@@ -1564,18 +1564,6 @@ int hg_coupling_factors(const int64_t *art_c, const double *art_a, int32_t na, c
 // ================================================================ stepping
 namespace {
 
-// The run-encoded variants (8..14) step only domains that have a run encoding, in a shape
-// of their own; a launch over any other domain takes the table form of the same variant.
-CollideCfg collide_cfg(const hg_ctx *ctx, bool runs, int parity, bool one_domain) {
-    CollideCfg cfg{ctx->storage, ctx->scheme, ctx->block, ctx->spt, ctx->variant};
-    if (cfg.variant >= 8 && !runs)
-        cfg.variant = cfg.variant == 8 || cfg.variant == 12 || cfg.variant == 13 ? 3
-                      : cfg.variant == 9                                      ? 5
-                      : cfg.variant == 10 || cfg.variant == 14                ? 6
-                                                                              : 7;
-    return run_cfg(cfg, parity, one_domain);
-}
-
 int build_plan(hg_ctx *ctx, const std::vector<int32_t> &doms, Plan *&out) {
     PlanKey key{doms};
     auto it = ctx->plans.find(key);
@@ -1611,8 +1599,8 @@ int build_plan(hg_ctx *ctx, const std::vector<int32_t> &doms, Plan *&out) {
     }
     for (size_t j = 0; j < doms.size(); ++j)
         if (!separate[j]) p->tiles_runs = p->tiles_runs && ctx->doms[doms[j]]->n_runs > 0;
-    const CollideCfg tcfg = collide_cfg(ctx, p->tiles_runs, 0, false);
-    const int64_t ts = (int64_t)tcfg.block * tcfg.spt;  // the same for every parity
+    const CollideCfg tcfg = collide_cfg(ctx->storage, ctx->scheme, 0, p->tiles_runs, false);
+    const int64_t ts = (int64_t)tcfg.block * tcfg.spt;  // kTile, whatever the parity
     for (size_t j = 0; j < doms.size(); ++j) {
         const int32_t di = doms[j];
         hg_domain *d = ctx->doms[di];
@@ -1797,7 +1785,7 @@ cudaError_t launch_sc(hg_ctx *ctx, Plan *p, int off, int parity, bool overlap) {
     bool chained = overlap;
     auto one_domain = [&](const DomDev &D, int64_t n) {
         if (n == 0) return cudaSuccess;
-        const CollideCfg cfg = collide_cfg(ctx, D.lword != nullptr, parity, true);
+        const CollideCfg cfg = collide_cfg(ctx->storage, ctx->scheme, parity, D.lword != nullptr, true);
         const int64_t ts = (int64_t)cfg.block * cfg.spt;
         const OneDomain one{&D, n, steps, chained};
         chained = true;
@@ -1809,7 +1797,7 @@ cudaError_t launch_sc(hg_ctx *ctx, Plan *p, int off, int parity, bool overlap) {
     }
     if (p->single) return one_domain(p->one, ctx->doms[p->doms[0]]->n);
     if (p->n_tiles == 0) return cudaSuccess;
-    return launch_stream_collide(collide_cfg(ctx, p->tiles_runs, parity, false), table, (const TileDev *)p->tiles.p,
+    return launch_stream_collide(collide_cfg(ctx->storage, ctx->scheme, parity, p->tiles_runs, false), table, (const TileDev *)p->tiles.p,
                                  p->n_tiles, off, parity, OneDomain{nullptr, 0, steps, chained}, ctx->stream);
 }
 
@@ -2482,7 +2470,7 @@ int split_plan(hg_split *sp, Plan *&out) {
     std::unique_ptr<Plan> p(new Plan);
     p->doms = key.doms;
     for (const SplitPart &P : sp->parts) p->tiles_runs = p->tiles_runs && P.n_runs > 0;
-    const CollideCfg tcfg = collide_cfg(ctx, p->tiles_runs, 2, false);
+    const CollideCfg tcfg = collide_cfg(ctx->storage, ctx->scheme, 2, p->tiles_runs, false);
     const int64_t ts = (int64_t)tcfg.block * tcfg.spt;
     std::vector<TileDev> tiles;
     for (const SplitPart &P : sp->parts) {

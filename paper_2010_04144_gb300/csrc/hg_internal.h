@@ -105,35 +105,36 @@ struct IoDev {
 // Slots reduced by one CTA of the iolet-update kernel.
 constexpr int kIoChunk = 256;
 
-// Launch configuration of the stream-collide kernel.
+// Launch configuration of the stream-collide kernel: the run-encoded form wherever the
+// launch's domains have one, else the 18-row table's, in the shape measured best on the
+// ~10M-site tree (us; threads x sites per thread).
+//   runs:  FP32 A/B 256 x 2 236, 128 x 2 243,
+//          256 x 1 246, 512 x 2 246; 16-bit A/B 256 x 1 178, 128 x 1 190, 256 x 2 182, 512 x 1
+//          190; AA odd 128 x 1 268 (FP32) and 197 (FP16), 256 x 1 274 and 203, 128 x 2 307 and
+//          236 (64 registers against 40)
+//   table: FP32 A/B 256 x 1 320 (rows) and 330 (Morton), 128 x 1 322 and 337, 256 x 2 325 and
+//          340; 16-bit A/B pairs 128 x 2 221 and 228, 256 x 2 224 and 231; AA odd 256 x 1 340
+//          and 429 (FP32), 128 x 1 338 and 435, 512 x 1 346 and 432
+//   AA even (site pairs): 128 x 2 222 (FP32) and 118 (FP16), 256 x 2 225 and 125
+// What the run form gains in rows ordering: FP32 A/B 236 against 320, FP16 A/B 178 / 221, AA
+// odd 268 / 340 and 197 / 260.  A tile table serves odd and even launches alike: its tiles hold
+// kTile sites.
 struct CollideCfg {
     int storage;
     int scheme;
+    bool runs;
     int block;
     int spt;
-    int variant;  // 0 = gathers into registers, 1 = gathers staged by cp.async (spt 1 or 2),
-                  // 2 = as 1, and the AA even step moves whole rows with TMA bulk copies,
-                  // 3 = as 0 with L2 prefetch hints, 4 = as 1 with the AA odd step's
-                  // stores staged in shared memory (spt 1), 5 = A/B on adjacent site
-                  // pairs (16-bit storage, spt 2), 6 / 7 = AA on adjacent site pairs (spt 2,
-                  // 7 with hints), 8..14 = the run encoding, in the shape of run_cfg
 };
-
-// Launch shape of the run-encoded kernel.  Measured on the ~10M-site tree (us): FP32 A/B 256 x 2
-// 241, 128 x 2 243, 256 x 1 246, 512 x 2 246; 16-bit A/B 256 x 1 181, 128 x 1 190, 256 x 2 182,
-// 512 x 1 190; AA odd 128 x 1 272 (FP32) and 198 (FP16), 256 x 1 274 and 203, 128 x 2 307 and
-// 236 (64 registers against 40); AA even (site pairs) 128 x 2 225 and 123, 256 x 2 225 and 125.
-// A tile table serves odd and even launches alike: its tiles hold 256 sites.
-constexpr int kRunTile = 256;
-__host__ __device__ constexpr int run_spt(int storage, int scheme, int parity) {
-    return scheme == kAB ? (storage == kF32 ? 2 : 1) : (parity == 1 ? 1 : 2);
+constexpr int kTile = 256;
+__host__ __device__ constexpr int sc_spt(int storage, int scheme, int parity, bool runs) {
+    return scheme == kAB ? ((storage == kF32) == runs ? 2 : 1) : (parity == 1 ? 1 : 2);
 }
-inline CollideCfg run_cfg(CollideCfg cfg, int parity, bool one_domain) {
-    if (cfg.variant < 8) return cfg;
-    cfg.spt = run_spt(cfg.storage, cfg.scheme, parity);
-    cfg.block = kRunTile / cfg.spt;
-    if (one_domain && cfg.scheme == kAB && cfg.storage == kF32) cfg.block = 256;
-    if (one_domain && cfg.scheme == kAA) cfg.block = 128;
+inline CollideCfg collide_cfg(int storage, int scheme, int parity, bool runs, bool one_domain) {
+    CollideCfg cfg{storage, scheme, runs, 0, sc_spt(storage, scheme, parity, runs)};
+    cfg.block = kTile / cfg.spt;
+    if (one_domain && runs && scheme == kAB && storage == kF32) cfg.block = 256;
+    if (one_domain && runs && scheme == kAA) cfg.block = 128;
     return cfg;
 }
 
@@ -144,7 +145,7 @@ cudaError_t launch_stream_collide(const CollideCfg &cfg, const DomDev *doms, con
                                   cudaStream_t st);
 // The stream-collide kernels of one storage type S (0 f32, 1 f16, 2 bf16), scheme
 // (0 A/B, 1 AA) and launch parity PAR (0 even, 1 odd, 2 read from the step counter;
-// A/B always 2): every variant and shape, instantiated in a translation unit of its
+// A/B always 2), instantiated in a translation unit of its
 // own (hg_sc_part.cu, compiled once per combination, so the twelve build in parallel).
 template <int S, int SCHEME, int PAR>
 cudaError_t launch_sc_part(const CollideCfg &cfg, const DomDev *doms, const TileDev *tiles, int64_t n_tiles,

@@ -427,8 +427,7 @@ cudaError_t launch_stream_collide(const CollideCfg &cfg, const DomDev *doms, con
                                   int64_t n_tiles, int off, int parity, const OneDomain &one,
                                   cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
-    // A/B reads its buffer parity per block: specialising it measured slower (the
-    // compile-time buffer choice raised the variant-3 kernel from 52 to 58 registers)
+    // A/B reads its buffer parity per block (from the step counter)
     const int par = cfg.scheme == kAB ? 2 : (parity == 0 || parity == 1 ? parity : 2);
 #define HG_PART(S_, C_, P_)                                                                    \
     if (cfg.storage == S_ && cfg.scheme == C_ && par == P_)                                   \

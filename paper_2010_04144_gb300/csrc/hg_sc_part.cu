@@ -14,7 +14,8 @@ template <>
 cudaError_t launch_sc_part<HG_PART_S, HG_PART_SCHEME, HG_PART_PAR>(const CollideCfg &cfg, const DomDev *doms,
                                                                    const TileDev *tiles, int64_t n_tiles, int off,
                                                                    const OneDomain &one, cudaStream_t st) {
-    return launch_sc_spt<HG_PART_S, HG_PART_SCHEME, HG_PART_PAR>(cfg, doms, tiles, n_tiles, off, one, st);
+    return cfg.runs ? launch_sc<HG_PART_S, HG_PART_SCHEME, HG_PART_PAR, true>(cfg, doms, tiles, n_tiles, off, one, st)
+                    : launch_sc<HG_PART_S, HG_PART_SCHEME, HG_PART_PAR, false>(cfg, doms, tiles, n_tiles, off, one, st);
 }
 
 }  // namespace hg

@@ -5,6 +5,7 @@
 
 namespace hg {
 
+constexpr uint32_t kWaitLimit = 1u << 22;  // polls after which a wait gives up (seconds)
 constexpr int kStepsThreads = 512;  // most threads per block
 constexpr int kStepsPerSm = 3;      // blocks of that size per SM (links in shared memory: 40 registers; else 2)
 constexpr int kStepsTiles = 8;      // most tiles a site block owns

@@ -1,5 +1,5 @@
-"""The run-encoded stream-collide kernel against the 18-row table form, bit for bit, where its
-tiles end: site counts around multiples of its tiles, runs that end anywhere, sites with iolet
+"""The run-encoded stream-collide kernel against the 18-row table's, bit for bit, where their
+tiles end: site counts around multiples of the tiles, runs that end anywhere, sites with iolet
 links, every storage and scheme, one domain per launch and domains of mixed parity in one."""
 import numpy as np
 import pytest
@@ -40,33 +40,39 @@ def _geometries():
 
 @pytest.mark.parametrize("scheme", ["ab", "aa"])
 @pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
-def test_run_kernel_tile_edges(gpu, storage, scheme):
+def test_run_and_table_kernels_tile_edges(gpu, storage, scheme):
+    """Rows ordering has runs, Morton ordering none: the two kernels on the same state."""
     for geo in _geometries():
         got = []
-        for variant, spt in ((0, 1), (8, 1)):
-            ctx = gpu.Context(storage=storage, scheme=scheme, kernel_variant=variant, sites_per_thread=spt)
-            d = ctx.domain(geo.xyz, geo.iolets, ordering="rows")
-            assert d.info()["n_runs"] > 0
+        for ordering in ("rows", "morton"):
+            ctx = gpu.Context(storage=storage, scheme=scheme)
+            d = ctx.domain(geo.xyz, geo.iolets, ordering=ordering)
+            assert (d.info()["n_runs"] > 0) == (ordering == "rows")
             d.load_state(_state(d, 3))
-            ctx.step(5)
+            ctx.step_profiled(5)  # one launch per step, whatever the size of the set
             got.append((d.state().copy(), d.iolet_stats(), d.boundary_values()))
             ctx.close()
         for a, b in zip(*got):
             assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("scheme", ["ab", "aa"])
 @pytest.mark.parametrize("storage", ["f32", "f16"])
-def test_run_kernel_mixed_parity_launch(gpu, storage):
+def test_packed_and_mixed_parity_launches(gpu, storage, scheme):
+    """Several domains in one launch, at the same and at different step parities, with and
+    without runs (one domain without them takes the whole launch to the table form)."""
     geos = [S.tree(S.TreeSpec(depth=3, scale=s)) for s in (0.3, 0.35, 0.4)]
     got = []
-    for variant, spt in ((0, 1), (14, 2)):
-        ctx = gpu.Context(storage=storage, scheme="aa", kernel_variant=variant, sites_per_thread=spt, block_size=128)
-        doms = [ctx.domain(g.xyz, g.iolets, ordering="rows") for g in geos]
+    for orderings in (("rows",) * 3, ("morton",) * 3, ("rows", "morton", "rows")):
+        ctx = gpu.Context(storage=storage, scheme=scheme)
+        doms = [ctx.domain(g.xyz, g.iolets, ordering=o) for g, o in zip(geos, orderings)]
         for j, d in enumerate(doms):
             d.load_state(_state(d, 5 + j))
+        ctx.step_profiled(3)
         ctx.step_domains(doms[:1], 1)
-        ctx.step_domains(doms, 7)
+        ctx.step_profiled(7)
         got.append([d.state().copy() for d in doms])
         ctx.close()
-    for a, b in zip(*got):
-        assert np.array_equal(a, b)
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.array_equal(a, b)
