@@ -64,7 +64,6 @@ template <> struct St<kF32> {
     template <int I> static __device__ __forceinline__ float ld(T v) { return v; }
     template <int I> static __device__ __forceinline__ T st(float v) { return v; }
     template <int I> static __device__ __forceinline__ float phys(T v) { return v; }
-    static __device__ __forceinline__ double ldd(T v, int) { return (double)v; }
 };
 template <> struct St<kF16> {
     using T = __half;
@@ -72,7 +71,6 @@ template <> struct St<kF16> {
     template <int I> static __device__ __forceinline__ float ld(T v) { return __half2float(v); }
     template <int I> static __device__ __forceinline__ T st(float v) { return __float2half_rn(v); }
     template <int I> static __device__ __forceinline__ float phys(T v) { return mulw<I>(__half2float(v)); }
-    static __device__ __forceinline__ double ldd(T v, int i) { return __dmul_rn((double)__half2float(v), WD(i)); }
 };
 template <> struct St<kBF16> {
     using T = __nv_bfloat16;
@@ -80,7 +78,6 @@ template <> struct St<kBF16> {
     template <int I> static __device__ __forceinline__ float ld(T v) { return __bfloat162float(v); }
     template <int I> static __device__ __forceinline__ T st(float v) { return __float2bfloat16_rn(v); }
     template <int I> static __device__ __forceinline__ float phys(T v) { return mulw<I>(__bfloat162float(v)); }
-    static __device__ __forceinline__ double ldd(T v, int i) { return __dmul_rn((double)__bfloat162float(v), WD(i)); }
 };
 
 template <int N> struct IC { static constexpr int v = N; };

@@ -236,87 +236,106 @@ __global__ void __launch_bounds__(128) k_guo_force(const DomDev *__restrict__ do
     D.bnd[slot] = mf;
 }
 
-// ---- read-back: F_t of site s, direction I (raw storage value) ----
-template <int S, int SCHEME, int I>
-__device__ __forceinline__ typename St<S>::T stored_F(const DomDev &D, int64_t t, int64_t s) {
+// ---- read-back: where F_t of a site is stored ----
+// Four arrangements: A/B in the buffer of t's parity; AA after an even step swapped at the own
+// site; AA after an odd step at x + c_I (or raw at the own site), found through the run encoding
+// or the 18-row table.  A kernel picks its arrangement once, outside its loop over sites: with
+// the choice inside, per value, the AA forms took 80-112 registers and one load at a time
+// (~10M-site tree in rows, fields: FP16 AA 443 -> 168 us after even steps, 763 -> 164 after odd
+// ones; FP32 AA 179 -> 184 and 497 -> 189; capped at 40 registers they spill: 190 and 254).
+enum Stored : int { kStoredAB, kStoredEven, kStoredOddRuns, kStoredOddTable };
+// f(IC<I>, place) for I = 0..18 in any order.
+template <int S, int KIND, typename F>
+__device__ __forceinline__ void each_stored(const DomDev &D, typename St<S>::T *buf, int64_t s, F &&f) {
     using T = typename St<S>::T;
-    const int64_t np = D.np;
-    if constexpr (SCHEME == kAB) {
-        return ((const T *)D.f[t & 1])[(int64_t)I * np + s];
+    const uint32_t npb = (uint32_t)D.np * sizeof(T);
+    T *p = buf + s;
+    if constexpr (KIND == kStoredAB) {
+        unroll<0, 19>([&](auto ic) { f(ic, row_at<decltype(ic)::v>(p, npb)); });
+    } else if constexpr (KIND == kStoredEven) {
+        unroll<0, 19>([&](auto ic) { f(ic, row_at<OPP(decltype(ic)::v)>(p, npb)); });
     } else {
-        const T *buf = (const T *)D.f[0];
-        if (!(t & 1) || I == 0) return buf[(int64_t)OPP(I) * np + s];
-        return buf[(int64_t)I * np + D.nbr[(int64_t)(OPP(I) - 1) * np + s]];  // x + c_I, or own raw
+        f(IC<0>{}, p);
+        auto link = [&](auto ic, int32_t off) {  // direction J lies where the gather of its opposite reads
+            constexpr int J = OPP(decltype(ic)::v);
+            f(IC<J>{}, pair_row<J>(p, npb) + off);
+        };
+        if constexpr (KIND == kStoredOddRuns) RunOffsets<kAA>{run_site(D, s), (int32_t)D.np}.each(link);
+        else TableOffsets<kAA, false>{D.nbr + s, (int32_t)s, (int32_t)D.np}.each(link);
     }
 }
-
-template <int S, int SCHEME, int I>
-__device__ __forceinline__ typename St<S>::T *stored_F_ptr(const DomDev &D, int64_t t, int64_t s) {
+// go(kind, buffer) with the arrangement of the domain after t steps.
+template <int S, int SCHEME, typename F>
+__device__ __forceinline__ void with_stored(const DomDev &D, int64_t t, F &&go) {
     using T = typename St<S>::T;
-    const int64_t np = D.np;
     if constexpr (SCHEME == kAB) {
-        return ((T *)D.f[t & 1]) + (int64_t)I * np + s;
+        go(IC<kStoredAB>{}, (T *)D.f[t & 1]);
     } else {
         T *buf = (T *)D.f[0];
-        if (!(t & 1) || I == 0) return buf + (int64_t)OPP(I) * np + s;
-        return buf + ((int64_t)I * np + D.nbr[(int64_t)(OPP(I) - 1) * np + s]);
+        if (!(t & 1)) go(IC<kStoredEven>{}, buf);
+        else if (D.lword) go(IC<kStoredOddRuns>{}, buf);
+        else go(IC<kStoredOddTable>{}, buf);
     }
 }
 
 template <int S, int SCHEME>
-__global__ void k_macroscopic(const DomDev *__restrict__ dd, int64_t n, const int32_t *canon_of,
-                              float4 *out) {
+__global__ void __launch_bounds__(256) k_macroscopic(const DomDev *__restrict__ dd, int64_t n,
+                                                     const int32_t *canon_of, float4 *out) {
     using Tr = St<S>;
-    const DomDev D = *dd;
-    const int64_t t = *D.step;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * blockDim.x) {
-        float g[19];
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            g[I] = Tr::template phys<I>(stored_F<S, SCHEME, I>(D, t, s));
-        });
-        float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            drho += g[I];
-            if (CX(I)) jx += CX(I) * g[I];
-            if (CY(I)) jy += CY(I) * g[I];
-            if (CZ(I)) jz += CZ(I) * g[I];
-        });
-        const float inv = 1.0f / (1.0f + drho);
-        out[canon_of ? canon_of[s] : s] = make_float4(drho, jx * inv, jy * inv, jz * inv);
-    }
+    const DomDev &D = *dd;
+    with_stored<S, SCHEME>(D, *D.step, [&](auto kc, typename Tr::T *buf) {
+        for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
+             s += (int64_t)gridDim.x * blockDim.x) {
+            float g[19];
+            each_stored<S, decltype(kc)::v>(D, buf, s, [&](auto ic, const typename Tr::T *at) {
+                constexpr int I = decltype(ic)::v;
+                g[I] = Tr::template phys<I>(*at);
+            });
+            float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
+            unroll<0, 19>([&](auto ic) {
+                constexpr int I = decltype(ic)::v;
+                drho += g[I];
+                if (CX(I)) jx += CX(I) * g[I];
+                if (CY(I)) jy += CY(I) * g[I];
+                if (CZ(I)) jz += CZ(I) * g[I];
+            });
+            const float inv = 1.0f / (1.0f + drho);
+            out[canon_of ? canon_of[s] : s] = make_float4(drho, jx * inv, jy * inv, jz * inv);
+        }
+    });
 }
 
 template <int S, int SCHEME>
-__global__ void k_export_state(const DomDev *__restrict__ dd, int64_t n, const int32_t *canon_of,
-                               typename St<S>::T *out, int64_t row) {
-    const DomDev D = *dd;
-    const int64_t t = *D.step;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = canon_of ? canon_of[s] : s;
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            out[(int64_t)I * row + c] = stored_F<S, SCHEME, I>(D, t, s);
-        });
-    }
+__global__ void __launch_bounds__(256) k_export_state(const DomDev *__restrict__ dd, int64_t n,
+                                                      const int32_t *canon_of, typename St<S>::T *out, int64_t row) {
+    using T = typename St<S>::T;
+    const DomDev &D = *dd;
+    with_stored<S, SCHEME>(D, *D.step, [&](auto kc, T *buf) {
+        for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
+             s += (int64_t)gridDim.x * blockDim.x) {
+            const int64_t c = canon_of ? canon_of[s] : s;
+            each_stored<S, decltype(kc)::v>(D, buf, s, [&](auto ic, const T *at) {
+                out[(int64_t)decltype(ic)::v * row + c] = *at;
+            });
+        }
+    });
 }
 
 template <int S, int SCHEME>
-__global__ void k_import_state(const DomDev *__restrict__ dd, int64_t n, const int32_t *canon_of,
-                               const typename St<S>::T *in, int64_t row) {
-    const DomDev D = *dd;
-    const int64_t t = *D.step;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = canon_of ? canon_of[s] : s;
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            *stored_F_ptr<S, SCHEME, I>(D, t, s) = in[(int64_t)I * row + c];
-        });
-    }
+__global__ void __launch_bounds__(256) k_import_state(const DomDev *__restrict__ dd, int64_t n,
+                                                      const int32_t *canon_of, const typename St<S>::T *in,
+                                                      int64_t row) {
+    using T = typename St<S>::T;
+    const DomDev &D = *dd;
+    with_stored<S, SCHEME>(D, *D.step, [&](auto kc, T *buf) {
+        for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
+             s += (int64_t)gridDim.x * blockDim.x) {
+            const int64_t c = canon_of ? canon_of[s] : s;
+            T v[19];  // all read before the first write: the loads are in flight together
+            unroll<0, 19>([&](auto ic) { v[decltype(ic)::v] = ldg_nc(in + (int64_t)decltype(ic)::v * row + c); });
+            each_stored<S, decltype(kc)::v>(D, buf, s, [&](auto ic, T *at) { *at = v[decltype(ic)::v]; });
+        }
+    });
 }
 
 // ---- halo exchange of a split domain (A/B scheme: F_t sits in f[t & 1]) ----
@@ -363,26 +382,53 @@ constexpr int kMassThreads = 256;
 // function of the state F_t alone: the same bits for A/B and AA and for every
 // device ordering.  Explicit rounding intrinsics keep every operation's order
 // fixed against compiler contraction.
+//
+// Bound by the FP64 unit (two operations per clock and SM): besides the product with the
+// weight (16-bit storage) and the addition, the FP32 -> FP64 conversion and the finiteness test
+// used to go there too; both are integer work on the FP32 bits here (~10M-site tree: FP32 1459
+// -> 794 us, FP16 1818 -> 1125).
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f), e = b & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (double)f;  // zero, subnormal, Inf, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+struct MassSum {
+    double a = 0.0;
+    int bad = 0;
+    template <int S> __device__ __forceinline__ void add(const float g[19]) {  // stored values, direction order
+        unroll<0, 19>([&](auto ic) {
+            constexpr int I = decltype(ic)::v;
+            const double v = widen(g[I]);
+            a = __dadd_rn(a, St<S>::kScaled ? __dmul_rn(v, WD(I)) : v);
+            bad += (__float_as_uint(g[I]) & 0x7f800000u) == 0x7f800000u;
+        });
+    }
+    __device__ __forceinline__ void finish(double2 *out) {
+        double b = (double)bad;
+        block_sum2(a, b);
+        if (threadIdx.x == 0) *out = make_double2(a, b);
+    }
+};
 template <int S, int SCHEME>
 __global__ void __launch_bounds__(kMassThreads) k_mass_partials(const DomDev *__restrict__ dd,
                                                                 int64_t n, const int32_t *dev_of,
                                                                 double2 *partials) {
-    const DomDev D = *dd;
-    const int64_t t = *D.step;
+    using Tr = St<S>;
+    const DomDev &D = *dd;
     const int64_t lo = (int64_t)blockIdx.x * kMassChunk;
     const int64_t hi = lo + kMassChunk < n ? lo + kMassChunk : n;
-    double a = 0.0, b = 0.0;
-    for (int64_t c = lo + threadIdx.x; c < hi; c += blockDim.x) {
-        const int64_t s = dev_of ? (int64_t)dev_of[c] : c;
-        unroll<0, 19>([&](auto ic) {
-            constexpr int I = decltype(ic)::v;
-            const double v = St<S>::ldd(stored_F<S, SCHEME, I>(D, t, s), I);
-            a = __dadd_rn(a, v);
-            if (!isfinite(v)) b = __dadd_rn(b, 1.0);
-        });
-    }
-    block_sum2(a, b);
-    if (threadIdx.x == 0) partials[blockIdx.x] = make_double2(a, b);
+    MassSum sum;
+    with_stored<S, SCHEME>(D, *D.step, [&](auto kc, typename Tr::T *buf) {
+        for (int64_t c = lo + threadIdx.x; c < hi; c += blockDim.x) {
+            const int64_t s = dev_of ? (int64_t)dev_of[c] : c;
+            float g[19];
+            each_stored<S, decltype(kc)::v>(D, buf, s, [&](auto ic, const typename Tr::T *at) {
+                g[decltype(ic)::v] = Tr::template ld<decltype(ic)::v>(*at);
+            });
+            sum.template add<S>(g);
+        }
+    });
+    sum.finish(partials + blockIdx.x);
 }
 
 // The same sum over a state already in canonical order ([19][stride]).
@@ -391,17 +437,16 @@ __global__ void __launch_bounds__(kMassThreads) k_mass_partials_flat(const typen
                                                                      int64_t stride, double2 *partials) {
     const int64_t lo = (int64_t)blockIdx.x * kMassChunk;
     const int64_t hi = lo + kMassChunk < n ? lo + kMassChunk : n;
-    double a = 0.0, b = 0.0;
+    MassSum sum;
     for (int64_t c = lo + threadIdx.x; c < hi; c += blockDim.x) {
+        float g[19];
         unroll<0, 19>([&](auto ic) {
             constexpr int I = decltype(ic)::v;
-            const double v = St<S>::ldd(f[(int64_t)I * stride + c], I);
-            a = __dadd_rn(a, v);
-            if (!isfinite(v)) b = __dadd_rn(b, 1.0);
+            g[I] = St<S>::template ld<I>(f[(int64_t)I * stride + c]);
         });
+        sum.template add<S>(g);
     }
-    block_sum2(a, b);
-    if (threadIdx.x == 0) partials[blockIdx.x] = make_double2(a, b);
+    sum.finish(partials + blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kMassThreads) k_mass_final(const double2 *partials, int64_t np_,
