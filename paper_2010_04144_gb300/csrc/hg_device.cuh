@@ -598,15 +598,10 @@ __device__ __forceinline__ void tile_aa_even_pairs(const DomDev &D, const TileDe
 }
 
 // ==== one site per thread: the A/B step and the AA odd step ====================
-// With the run encoding -- what bounds it: for 16-bit storage instruction issue (68 % of the slots; 438 instructions
-// per site and A/B step, 518 before the links were decoded as below), for FP32 HBM (A/B) and
-// the misaligned scatter (AA odd).  40 registers, so 48 warps per SM hide the chain word ->
-// run row -> gathers.  ~10M-site tree, stream-collide alone, before -> now: FP32 A/B 243 ->
-// 236 us, FP16 A/B 192 -> 178, FP32 AA odd 303 -> 268, FP16 AA odd 236 -> 197 (even 119).
-// Tried and slower: two sites per thread with packed arithmetic (350 instructions per site,
-// but 64-90 registers: 188-230 us FP16 A/B); lists of all-fluid pairs and single sites (250
-// instructions per site, but the lists' stores leave sectors half written: FP32 A/B 296 us);
-// an L2 prefetch of the rows 64K..1M sites ahead (no change to 20 % slower).
+// ==== one site per thread: the A/B step and the AA odd step ====================
+// FP32 AA odd through the run encoding: bound by the misaligned scatter's sectors (268 us on the
+// ~10M-site tree, 303 before the links were decoded as below); 40 registers, so 48 warps per SM
+// hide the chain word -> run row -> gathers.
 // With the 18-row table it is bound by the table's 72 bytes and the scattered sectors of
 // Morton order (~10M-site tree, Morton / rows): FP32 A/B 330 / 320 us (475 before the 32-bit
 // multiply-add addresses), FP16 AA odd 343 / 260 and FP32 AA odd 429 / 340, against 391 / 346
@@ -656,10 +651,10 @@ template <int SCHEME, bool HINT> struct TableOffsets {
 };
 // A/B step or AA odd step of one site.  The AA scatter goes to the places the gather read
 // (direction I where its opposite was read); their 18 offsets wait in shared memory, one bank
-// per thread (`stash`: this thread's), instead of being decoded again.
+// per thread (`stash`: this thread's, a word per `stride`), instead of being decoded again.
 template <int S, int SCHEME, bool HINT, typename L>
 __device__ __forceinline__ void site_links(const DomDev &D, const typename St<S>::T *src, typename St<S>::T *dst,
-                                           int64_t s, const L &links, int32_t *stash) {
+                                           int64_t s, const L &links, int32_t *stash, int stride) {
     using Tr = St<S>;
     using T = typename Tr::T;
     const uint32_t npb = (uint32_t)D.np * sizeof(T);
@@ -669,7 +664,7 @@ __device__ __forceinline__ void site_links(const DomDev &D, const typename St<S>
     links.each([&](auto ic, int32_t off) {
         constexpr int I = decltype(ic)::v;
         g[I] = link_ld<S, SCHEME, HINT>(pair_row<I>(p, npb) + off);
-        if constexpr (SCHEME == kAA) stash[(I - 1) * blockDim.x] = off;
+        if constexpr (SCHEME == kAA) stash[(I - 1) * stride] = off;
     });
     int slot = -1;
     if (links.next_to_iolet(D, s)) {
@@ -690,35 +685,97 @@ __device__ __forceinline__ void site_links(const DomDev &D, const typename St<S>
         constexpr int I = decltype(ic)::v;
         const T v = Tr::template st<I>(g[I]);
         if constexpr (SCHEME == kAB) *row_at<I>(q, npb) = v;
-        else pair_row<I>(q, npb)[back[(OPP(I) - 1) * blockDim.x]] = v;
+        else pair_row<I>(q, npb)[back[(OPP(I) - 1) * stride]] = v;
     });
     if (slot >= 0) D.bnd[slot] = m;
 }
-// A tile of SPT * blockDim sites; with SPT = 2 both words are loaded, and both run rows
-// prefetched into L1 (80 bytes: at most two lines), before the first site's gathers.
-template <int S, int SCHEME, int SPT>
-__device__ __forceinline__ void tile_runs(const DomDev &D, const TileDev &tl, const typename St<S>::T *src,
-                                          typename St<S>::T *dst, int32_t *stash) {
-    RunSite r[SPT];
-#pragma unroll
-    for (int j = 0; j < SPT; ++j) {
-        const int q = j * blockDim.x + threadIdx.x;
-        r[j].w = 0;
-        r[j].row = D.rdelta;
-        if (q < tl.count) {
-            r[j] = run_site(D, tl.start + q);
-            if constexpr (SPT > 1) {
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(r[j].row));
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(r[j].row + kRunStride - 1));
-            }
+// ---- A/B step or 16-bit AA odd step of a pair of adjacent sites, run encoding ----
+// The A/B steps and the 16-bit AA odd step run near the issue limit one site per thread (420 to
+// 518 instructions per site and step).  A pair (s even) shares the word load, the run row where
+// the run is the same (98 % of the pairs), the rows' addresses, vector stores (A/B) and a packed
+// collision: 303 instructions per site for A/B, 390 for AA odd.  Registers decide: ~10M-site
+// tree, FP16 A/B at 76 / 72 / 64 / 56 registers 178 / 167 / 158 / 166 us (one site per thread
+// 178), FP16 AA odd at 85 / 72 / 64 213 / 190 / 200 (197).  Bound now by the latency of the
+// chain word -> row -> gathers at 28 warps per SM.
+// Tried and slower: sites l and l + 32 of a warp as the pair (188-230 us); lists of all-fluid
+// pairs and single sites (250 instructions per site, but their stores leave sectors half
+// written: FP32 A/B 296 us); an L2 prefetch of the distributions 64K..1M sites ahead (no change
+// to 20 % slower); joining the AA scatter's two stores where they meet (FP16 190 -> 211).
+template <int S, int SCHEME>
+__device__ __forceinline__ void site_run_pair(const DomDev &D, const typename St<S>::T *src,
+                                              typename St<S>::T *dst, int64_t s, int2 *stash) {
+    using Tr = St<S>;
+    using T = typename Tr::T;
+    const int32_t np = (int32_t)D.np;
+    const uint32_t npb = (uint32_t)D.np * sizeof(T);
+    const uint2 w = __ldg(reinterpret_cast<const uint2 *>(D.lword + s));
+    const int32_t r0 = __ldg(D.run0 + (s >> 10));
+    const int32_t *ra = D.rdelta + (int64_t)(r0 + (int32_t)((w.x >> 18) & 1023u)) * kRunStride;
+    const int32_t *rb = D.rdelta + (int64_t)(r0 + (int32_t)((w.y >> 18) & 1023u)) * kRunStride;
+    const bool same = ra == rb;
+    const T *p = src + s;
+    F2 g[19];
+    g[0] = ld_pair<S, 0>(p);
+    unroll<0, 5>([&](auto kc) {
+        constexpr int K = decltype(kc)::v;
+        const int4 va = __ldg(reinterpret_cast<const int4 *>(ra) + K);
+        int4 vb = va;
+        if (!same) vb = __ldg(reinterpret_cast<const int4 *>(rb) + K);
+        const int32_t da[4] = {va.x, va.y, va.z, va.w}, db[4] = {vb.x, vb.y, vb.z, vb.w};
+        unroll<0, (K < 4 ? 4 : 2)>([&](auto jc) {
+            constexpr int J = decltype(jc)::v, I = 4 * K + J + 1;
+            const T *q = pair_row<I>(p, npb);
+            const int32_t oa = run_offset<SCHEME, I>(w.x, da[J], np), ob = run_offset<SCHEME, I>(w.y, db[J], np);
+            const float a = link_ld<S, SCHEME, true>(q + oa);
+            const float b = link_ld<S, SCHEME, true>(q + 1 + ob);
+            g[I] = pk2(a, b);
+            if constexpr (SCHEME == kAA) stash[(I - 1) * blockDim.x] = make_int2(oa, ob);
+        });
+    });
+    int slot_a = -1, slot_b = -1;
+    if ((w.x | w.y) >> 31) {
+        wait_for_iolet_update();
+        const uint32_t word = __ldg(D.iomask + (s >> 5));
+        if (w.x >> 31) {
+            slot_a = site_slot(D, s, word);
+            iolet_links_half<S, false>(D, D.bcv, slot_a, g);
+        }
+        if (w.y >> 31) {
+            slot_b = site_slot(D, s + 1, word);
+            iolet_links_half<S, true>(D, D.bcv, slot_b, g);
         }
     }
-#pragma unroll
-    for (int j = 0; j < SPT; ++j) {
-        const int q = j * blockDim.x + threadIdx.x;
-        if (q < tl.count)
-            site_links<S, SCHEME, true>(D, src, dst, tl.start + q, RunOffsets<SCHEME>{r[j], (int32_t)D.np}, stash);
-    }
+    const MomT<F2> m = collide_v<Tr::kScaled>(g, D.omega, D.neg_zero2);
+    int2 *back = stash;
+    if constexpr (SCHEME == kAA)
+        asm volatile("{\n\t.reg .b64 t;\n\tmov.b64 t, %2;\n\tmov.b64 %0, %1;\n\t}"
+                     : "=l"(back) : "l"(stash), "l"(m.drho.v) : "memory");
+    T *q = opaque(dst + s);
+    st_pair<S, 0>(q, g[0]);
+    unroll<1, 19>([&](auto ic) {
+        constexpr int I = decltype(ic)::v;
+        if constexpr (SCHEME == kAB) {
+            st_pair<S, I>(row_at<I>(q, npb), g[I]);
+        } else {
+            const int2 o = back[(OPP(I) - 1) * blockDim.x];
+            T *r = pair_row<I>(q, npb);
+            r[o.x] = Tr::template st<I>(lo2(g[I]));
+            r[1 + o.y] = Tr::template st<I>(hi2(g[I]));
+        }
+    });
+    put_moments(D, slot_a, slot_b, m);
+}
+
+constexpr int64_t kWordsAhead = 196608;  // sites
+
+// Launch bounds: the run-encoded pair forms are held to 64 (A/B) and 72 (AA odd) registers; the
+// others keep what 512 threads leave them, which they use least of (40 to 76).
+constexpr bool pair_runs(int s, int scheme, int par, bool runs) {
+    return runs && (scheme == kAB || (par == 1 && s != kF32));
+}
+constexpr int sc_threads(int s, int scheme, int par, bool runs) { return pair_runs(s, scheme, par, runs) ? 128 : 512; }
+constexpr int sc_blocks(int s, int scheme, int par, bool runs) {
+    return pair_runs(s, scheme, par, runs) ? (scheme == kAB ? 8 : 7) : 0;
 }
 
 // PAR is the parity of the step this launch executes: 0 = even, 1 = odd (the
@@ -742,13 +799,36 @@ __device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileD
     const T *src = (const T *)D.f[SCHEME == kAA || odd ? 0 : 1];  // A/B: F_{t-1} sits in f[(t-1) & 1]
     T *dst = (T *)D.f[SCHEME == kAA || !odd ? 0 : 1];
     if constexpr (RUNS) {
-        tile_runs<S, SCHEME, SPT>(D, tl, src, dst, stash);
+        if constexpr (SCHEME == kAB) {
+            // the words of a later tile into L2 (a line per thread): FP32 235 -> 231 us, FP16 158
+            // -> 156 at 128K..300K sites ahead, nothing at 1.2M; AA odd loses 3 %
+            const int64_t at = tl.start + kWordsAhead + 32 * (int64_t)threadIdx.x;
+            if (threadIdx.x < kTile / 32 && at < D.n) asm volatile("prefetch.global.L2 [%0];" ::"l"(D.lword + at));
+        }
+        constexpr bool PAIRS = pair_runs(S, SCHEME, PAR, true);
+        constexpr int WORDS = PAIRS ? 2 : 1;  // of shared memory per thread and link
+        auto one_site = [&](int64_t s) {
+            site_links<S, SCHEME, true>(D, src, dst, s, RunOffsets<SCHEME>{run_site(D, s), (int32_t)D.np},
+                                        stash + WORDS * threadIdx.x, WORDS * (int)blockDim.x);
+        };
+        if constexpr (PAIRS) {
+            const int r = 2 * threadIdx.x;  // even sites: tiles start at multiples of kTile
+            if (r + 1 < tl.count) site_run_pair<S, SCHEME>(D, src, dst, tl.start + r, (int2 *)stash + threadIdx.x);
+            else if (r < tl.count) one_site(tl.start + r);
+        } else {
+#pragma unroll
+            for (int j = 0; j < SPT; ++j) {
+                const int r = j * blockDim.x + threadIdx.x;
+                if (r < tl.count) one_site(tl.start + r);
+            }
+        }
     } else {
         // FP32 AA without the 256-byte hints: 429 us against 446 (Morton), 340 against 346 (rows)
         constexpr bool HINT = !(SCHEME == kAA && S == kF32);
         auto one_site = [&](int64_t s) {
             site_links<S, SCHEME, HINT>(D, src, dst, s,
-                                        TableOffsets<SCHEME, HINT>{D.nbr + s, (int32_t)s, (int32_t)D.np}, stash);
+                                        TableOffsets<SCHEME, HINT>{D.nbr + s, (int32_t)s, (int32_t)D.np},
+                                        stash + threadIdx.x, (int)blockDim.x);
         };
         if constexpr (SCHEME == kAB && S != kF32) {
             const int r = 2 * threadIdx.x;  // even sites: tiles start at multiples of kTile
@@ -768,9 +848,9 @@ __device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileD
 // first threads copy the tile's domain descriptor into shared memory, one
 // 8-byte word each, while thread 0 reads the domain's step counter.
 template <int S, int SCHEME, int PAR, bool RUNS>
-__global__ void __launch_bounds__(512) k_stream_collide(const DomDev *__restrict__ doms,
-                                                          const TileDev *__restrict__ tiles,
-                                                          const int64_t *__restrict__ steps, int off) {
+__global__ void __launch_bounds__(sc_threads(S, SCHEME, PAR, RUNS), sc_blocks(S, SCHEME, PAR, RUNS))
+    k_stream_collide(const DomDev *__restrict__ doms, const TileDev *__restrict__ tiles,
+                     const int64_t *__restrict__ steps, int off) {
     static_assert(sizeof(DomDev) % 8 == 0, "descriptor copied in 8-byte words");
     constexpr int kWords = (int)(sizeof(DomDev) / 8);
     __shared__ DomDev D;
@@ -786,14 +866,15 @@ __global__ void __launch_bounds__(512) k_stream_collide(const DomDev *__restrict
         if (threadIdx.x == 0) t_now = __ldg(steps + tl.dom) + off + 1;
     __syncthreads();
     const bool odd = PAR == 2 ? (t_now & 1) != 0 : PAR == 1;
-    stream_collide_tile<S, SCHEME, PAR, RUNS>(D, tl, odd, stash + threadIdx.x);
+    stream_collide_tile<S, SCHEME, PAR, RUNS>(D, tl, odd, stash);
 }
 
 // One domain per launch: the descriptor is a kernel parameter (constant bank)
 // and block b takes sites [b*T, b*T + T) with T = sites per thread * blockDim, so no
 // block waits on a table load or a barrier before its first neighbour-table load.
 template <int S, int SCHEME, int PAR, bool RUNS>
-__global__ void __launch_bounds__(512) k_stream_collide_one(const __grid_constant__ DomDev D, int64_t n, int off) {
+__global__ void __launch_bounds__(sc_threads(S, SCHEME, PAR, RUNS), sc_blocks(S, SCHEME, PAR, RUNS))
+    k_stream_collide_one(const __grid_constant__ DomDev D, int64_t n, int off) {
     // a launch chained after this one (the next domain of a per-domain launch
     // sequence) may be scheduled once every block here has started; kernels launched
     // without programmatic serialisation ignore the trigger
@@ -807,7 +888,7 @@ __global__ void __launch_bounds__(512) k_stream_collide_one(const __grid_constan
     bool odd;
     if constexpr (PAR == 2) odd = ((__ldg(D.step) + off + 1) & 1) != 0;
     else odd = PAR == 1;
-    stream_collide_tile<S, SCHEME, PAR, RUNS>(D, tl, odd, stash + threadIdx.x);
+    stream_collide_tile<S, SCHEME, PAR, RUNS>(D, tl, odd, stash);
 }
 
 template <int S, int SCHEME, int PAR, bool RUNS>
@@ -816,8 +897,8 @@ cudaError_t launch_sc(const CollideCfg &cfg, const DomDev *doms, const TileDev *
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)n_tiles);
     lc.blockDim = dim3((unsigned)cfg.block);
-    // the AA odd step's 18 offsets per thread
-    lc.dynamicSmemBytes = SCHEME == kAA && PAR != 0 ? (size_t)18 * 4 * cfg.block : 0;
+    // the AA odd step's 18 offsets per thread (two sites' in the pair form)
+    lc.dynamicSmemBytes = SCHEME == kAA && PAR != 0 ? (size_t)18 * 4 * (PAR == 1 ? cfg.spt : 1) * cfg.block : 0;
     lc.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -108,16 +108,16 @@ constexpr int kIoChunk = 256;
 // Launch configuration of the stream-collide kernel: the run-encoded form wherever the
 // launch's domains have one, else the 18-row table's, in the shape measured best on the
 // ~10M-site tree (us; threads x sites per thread).
-//   runs:  FP32 A/B 256 x 2 236, 128 x 2 243,
-//          256 x 1 246, 512 x 2 246; 16-bit A/B 256 x 1 178, 128 x 1 190, 256 x 2 182, 512 x 1
-//          190; AA odd 128 x 1 268 (FP32) and 197 (FP16), 256 x 1 274 and 203, 128 x 2 307 and
-//          236 (64 registers against 40)
+//   runs:  A/B in adjacent pairs (64 registers) 128 x 2: FP32 231, FP16 157, 64 x 2 the same,
+//          256 x 2 239 and 164, one site per thread 235 and 178; AA odd FP32 one site per thread
+//          (40 registers) 128 x 1 268, 256 x 1 274, pairs 271; AA odd 16-bit pairs (72
+//          registers) 128 x 2 190, one site per thread 197
 //   table: FP32 A/B 256 x 1 320 (rows) and 330 (Morton), 128 x 1 322 and 337, 256 x 2 325 and
 //          340; 16-bit A/B pairs 128 x 2 221 and 228, 256 x 2 224 and 231; AA odd 256 x 1 340
 //          and 429 (FP32), 128 x 1 338 and 435, 512 x 1 346 and 432
 //   AA even (site pairs): 128 x 2 222 (FP32) and 118 (FP16), 256 x 2 225 and 125
-// What the run form gains in rows ordering: FP32 A/B 236 against 320, FP16 A/B 178 / 221, AA
-// odd 268 / 340 and 197 / 260.  A tile table serves odd and even launches alike: its tiles hold
+// What the run form gains in rows ordering: FP32 A/B 231 against 320, FP16 A/B 157 / 221, AA
+// odd 268 / 340 and 190 / 260.  A tile table serves odd and even launches alike: its tiles hold
 // kTile sites.
 struct CollideCfg {
     int storage;
@@ -128,12 +128,11 @@ struct CollideCfg {
 };
 constexpr int kTile = 256;
 __host__ __device__ constexpr int sc_spt(int storage, int scheme, int parity, bool runs) {
-    return scheme == kAB ? ((storage == kF32) == runs ? 2 : 1) : (parity == 1 ? 1 : 2);
+    return scheme == kAB ? (runs || storage != kF32 ? 2 : 1) : parity == 1 ? (runs && storage != kF32 ? 2 : 1) : 2;
 }
 inline CollideCfg collide_cfg(int storage, int scheme, int parity, bool runs, bool one_domain) {
     CollideCfg cfg{storage, scheme, runs, 0, sc_spt(storage, scheme, parity, runs)};
     cfg.block = kTile / cfg.spt;
-    if (one_domain && runs && scheme == kAB && storage == kF32) cfg.block = 256;
     if (one_domain && runs && scheme == kAA) cfg.block = 128;
     return cfg;
 }
