@@ -778,6 +778,15 @@ constexpr int sc_blocks(int s, int scheme, int par, bool runs) {
     return pair_runs(s, scheme, par, runs) ? (scheme == kAB ? 8 : 7) : 0;
 }
 
+// The last site of an odd-sized tile.  Not inlined: the single-site body beside the pair's cost
+// the pair registers (FP16 A/B 160 us against 155, FP16 AA odd 194 against 184).
+template <int S, int SCHEME>
+__device__ __noinline__ void tail_site(const DomDev &D, const typename St<S>::T *src, typename St<S>::T *dst,
+                                       int64_t s, int32_t *stash) {
+    site_links<S, SCHEME, true>(D, src, dst, s, RunOffsets<SCHEME>{run_site(D, s), (int32_t)D.np}, stash,
+                                2 * (int)blockDim.x);
+}
+
 // PAR is the parity of the step this launch executes: 0 = even, 1 = odd (the
 // AA step kind), 2 = read from the domain's step counter per block (A/B, and AA
 // batches whose domains are at different parities).  RUNS: the domain has a run
@@ -814,7 +823,7 @@ __device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileD
         if constexpr (PAIRS) {
             const int r = 2 * threadIdx.x;  // even sites: tiles start at multiples of kTile
             if (r + 1 < tl.count) site_run_pair<S, SCHEME>(D, src, dst, tl.start + r, (int2 *)stash + threadIdx.x);
-            else if (r < tl.count) one_site(tl.start + r);
+            else if (r < tl.count) tail_site<S, SCHEME>(D, src, dst, tl.start + r, stash + WORDS * threadIdx.x);
         } else {
 #pragma unroll
             for (int j = 0; j < SPT; ++j) {
