@@ -118,3 +118,33 @@ def test_resident_two_contexts_at_once(gpu):
     for k in range(2):
         for a, b in zip(alone[k], both[k]):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("scheme", ["ab", "aa"])
+def test_steps_under_stream_capture(gpu, scheme):
+    """A caller's capture records plain launches (no resident launch, no graph of the library's
+    own), chained as on the stream: replays give the bits of stepping."""
+    torch = pytest.importorskip("torch")
+    geos, pairs = _pair(0.3)
+    got = []
+    for captured in (True, False):
+        ctx = gpu.Context(storage="f32", scheme=scheme)
+        doms = [ctx.domain(g.xyz, g.iolets, ordering=o) for g, o in zip(geos, ("rows", "morton"))]
+        ctx.couple(doms[0], doms[1], pairs)
+        ctx.step(2)
+        if captured:
+            ctx.sync()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=ctx.stream):
+                ctx.step(4)
+            with torch.cuda.stream(ctx.stream):
+                for _ in range(6):
+                    g.replay()
+            ctx.sync()
+        else:
+            ctx.step(24)
+        got.append([d.state().copy() for d in doms] + [d.iolet_stats() for d in doms]
+                   + [d.boundary_values() for d in doms])
+        ctx.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
