@@ -1860,46 +1860,56 @@ cudaError_t steps_launch(const hg_ctx *ctx, const StepsArgs &a, const StepsShape
 }
 
 // Largest set (sites of all its domains) that is stepped by resident launches.  Time per step of
-// a tree of n sites, launch by launch / resident (us; the slower of Morton and rows ordering
-// against its resident time): 290k FP32 A/B 16.7 / 8.9, FP16 AA 17.9 / 10.9; 385k FP32 A/B
-// 17.7 / 10.7, FP16 AA 19.5 / 17.4 (links no longer fit shared memory with three blocks per
-// SM); 480k FP16 AA 19.8 / 22.0, FP32 AA 21.1 / 23.2; 630k FP32 A/B 23.3 / 19.2, FP16 A/B
-// 17.3 / 15.7; 770k FP32 A/B 26.8 / 26.7, FP16 A/B 18.2 / 18.3.
+// a tree of n sites, launch by launch / resident (us, Morton; rows): 290k FP32 A/B 17.1 / 8.9;
+// 18.0 / 8.7, FP16 AA 16.5 / 10.5; 16.9 / 8.6; 385k FP32 A/B 19.7 / 10.6; 18.6 / 9.8, FP16 AA
+// 17.8 / 14.7; 16.7 / 11.3; 480k FP16 AA 18.6 / 18.8; 17.5 / 17.5, FP32 AA 20.7 / 20.7; 18.4 /
+// 18.0; 630k FP32 A/B 27.1 / 25.9; 22.6 / 17.8, FP16 A/B 21.7 / 15.3; 19.4 / 13.9.
 int64_t resident_sites(const hg_ctx *ctx) { return ctx->scheme == HG_SCHEME_AB ? 700000 : 450000; }
 
-// The shape of a resident launch over domains of the given sizes; false: none fits.  The
-// smallest blocks that give every block one tile, else the fewest tiles per block.
+// The shape of a resident launch over domains of the given sizes; false: none fits.  Fewest
+// tiles per block, links in shared memory if they fit, then the block size that leaves the
+// fullest SM the fewest sites, the larger of equals (166k sites FP32 A/B: blocks of 512 put 1536
+// sites on some SMs and 1024 on others, 7.35 us per step; 384 puts 1152 on each, 6.1).  At most
+// three blocks per SM: every block takes part in the barrier (16 tubes at five blocks of 192
+// per SM 13.3 us, at two of 512 11.2).  A/B blocks of three and more tiles read their links
+// from memory (385k sites FP32 Morton: 10.6 us against 14.2 from shared memory, where only 27
+// warps per SM fit; AA the other way, 17.8 against 16.0).
 bool steps_shape(const hg_ctx *ctx, const std::vector<int64_t> &sizes, int n_ios, StepsShape &sh, int &n_site_blocks) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return false;
     // iolet blocks: up to a sixth of the SMs' worth, one iolet each where that is enough, and
-    // then up to three blocks per iolet taking its steps in turn
-    const int sets = std::max((n_ios + kStepsIolets - 1) / kStepsIolets, std::min(n_ios, sms / 6));
-    sh.groups = sets == 0 ? 1 : std::max(1, std::min(kStepsLag - 1, sms / 6 / sets));
-    const int n_io = sets * sh.groups;
+    // then up to three blocks per iolet taking its steps in turn; a few where more do not fit
+    const int least = std::max((n_ios + kStepsIolets - 1) / kStepsIolets, std::min(n_ios, 8));
+    const int most = std::max(least, std::min(n_ios, sms / 6));
     for (int own = 1; own <= kStepsTiles; ++own)
-        for (int threads = own == 1 ? 128 : kStepsThreads; threads <= kStepsThreads; threads *= 2) {
-            int64_t tiles = 0;
-            for (int64_t n : sizes) tiles += (n + threads - 1) / threads;
-            n_site_blocks = (int)((tiles + own - 1) / own);
-            for (const bool stash : {true, false}) {
-                const size_t smem = stash ? (size_t)own * kStashRows * 4 * threads : 0;
-                int per_sm = 0;
-                if (smem > 200 * 1024) continue;
-                if (steps_blocks(ctx, stash, threads, smem, &per_sm) != cudaSuccess) {
-                    cudaGetLastError();
-                    return false;
+        for (const bool other : {false, true})
+            for (const int sets : {most, least}) {
+                const bool stash = (own >= 3 && ctx->scheme == HG_SCHEME_AB) == other;
+                const int groups = sets == 0 ? 1 : std::max(1, std::min(kStepsLag - 1, sms / 6 / sets));
+                int64_t best = INT64_MAX;
+                for (int threads = 64; threads <= kStepsThreads; threads += 32) {
+                    int64_t tiles = 0;
+                    for (int64_t n : sizes) tiles += (n + threads - 1) / threads;
+                    const int64_t blocks = (tiles + own - 1) / own, total = blocks + sets * groups;
+                    const int64_t per_sm = (total + sms - 1) / sms, load = per_sm * threads * own;
+                    const size_t smem = stash ? (size_t)own * kStashRows * 4 * threads : 0;
+                    if (smem > (size_t)kStepsSmem || per_sm > kStepsPerSm || load > best) continue;
+                    int room = 0;
+                    if (steps_blocks(ctx, stash, threads, smem, &room) != cudaSuccess) {
+                        cudaGetLastError();
+                        return false;
+                    }
+                    if (per_sm > room) continue;
+                    best = load;
+                    n_site_blocks = (int)blocks;
+                    sh.threads = threads;
+                    sh.smem = smem;
+                    sh.stash = stash;
+                    sh.groups = groups;
+                    sh.grid = (int)total;
                 }
-                // small blocks: spread over the SMs rather than stacked on a few
-                const int64_t room = (int64_t)sms * std::min(per_sm, threads < kStepsThreads ? 2 : kStepsPerSm);
-                if (n_site_blocks + n_io > room) continue;
-                sh.threads = threads;
-                sh.smem = smem;
-                sh.stash = stash;
-                sh.grid = n_site_blocks + n_io;
-                return true;
+                if (best < INT64_MAX) return true;
             }
-        }
     return false;
 }
 

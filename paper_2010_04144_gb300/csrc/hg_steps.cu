@@ -8,8 +8,8 @@
 // resident for all the steps: most blocks own fixed tiles of sites and keep their links in
 // shared memory, a few blocks do the iolet work, and one grid barrier (1.4 us) ends each step.
 // Per step, launches -> resident: 4.5k sites FP32 A/B 11.4 -> 3.1 us, 13k FP32 AA 12.0 -> 2.8,
-// 166k FP32 A/B 15.0 -> 7.5, 16 tubes of 279k FP16 AA 21.9 -> 11.4, coupled pair of 339k FP16
-// AA 22.9 -> 12.6.  What bounds it now: the barrier and one round of L2 latencies up to ~50k
+// 166k FP32 A/B 15.0 -> 6.1, 16 tubes of 279k FP16 AA 21.9 -> 11.2, coupled pair of 339k FP16
+// AA 22.9 -> 11.2.  What bounds it now: the barrier and one round of L2 latencies up to ~50k
 // sites, then L2 traffic.
 //
 //   step j:  site blocks   stream-collide (moments of iolet sites -> ring[j mod lag]), then
@@ -381,8 +381,9 @@ __global__ void __launch_bounds__(kStepsThreads, STASH ? kStepsPerSm : 2) k_step
 
 template <bool STASH> cudaError_t blocks_per_sm(int threads, size_t smem, int *out) {
     auto k = k_steps<HG_PART_S, HG_PART_SCHEME, STASH>;
+    // one allowance for every shape: sets of several shapes may be stepped in turn
     cudaError_t e = cudaSuccess;
-    if (smem > 32 * 1024) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (STASH) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kStepsSmem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k, threads, smem);
     return e;
 }

@@ -10,6 +10,7 @@ constexpr int kStepsThreads = 512;  // most threads per block
 constexpr int kStepsPerSm = 3;      // blocks of that size per SM (links in shared memory: 40 registers; else 2)
 constexpr int kStepsTiles = 8;      // most tiles a site block owns
 constexpr int kStepsIolets = 8;     // most iolets an iolet block owns
+constexpr int kStepsSmem = 200 * 1024;  // most dynamic shared memory of a block
 constexpr int kStashRows = 20;      // words of shared memory per site: 18 links, boundary slot, its word
 constexpr int kStepsChunks = 16;    // iolet chunks summed at a time
 constexpr int kStepsLag = 4;        // steps the iolet means may trail the sites (boundary-moment buffers)

@@ -148,3 +148,22 @@ def test_steps_under_stream_capture(gpu, scheme):
         ctx.close()
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+def test_resident_shapes_in_turn(gpu):
+    """Sets of different launch shapes (much and little shared memory) stepped in turn."""
+    geos = [S.box(128, 64, 32), S.cylinder(radius=4, length=20), S.parallel_tubes(3, radius=5, length=40)]
+    ctxs = [gpu.Context(storage="f32", scheme="aa") for _ in geos]
+    doms = [c.domain(g.xyz, g.iolets) for c, g in zip(ctxs, geos)]
+    for n in (2, 3, 4):
+        for c in ctxs:
+            c.step(n)
+    for c, g, d in zip(ctxs, geos, doms):
+        c.sync()
+        ref = gpu.Context(storage="f32", scheme="aa")
+        r = ref.domain(g.xyz, g.iolets)
+        ref.step_profiled(9)
+        for a, b in zip(_snapshot([d]), _snapshot([r])):
+            assert np.array_equal(a, b)
+        ref.close()
+        c.close()
