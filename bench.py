@@ -144,16 +144,15 @@ class ClockSampler:
 
 
 def profiled_traffic(variant_key, launch, ordering="morton"):
-    """DRAM bytes per launch from the committed ncu summary, if it matches this kernel build,
-    launch shape and site ordering."""
+    """DRAM bytes per launch from the committed ncu summary, if it matches this kernel build
+    and site ordering (the library picks the launch shape itself)."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as f:
             t = json.load(f)
         entries = t.get(variant_key) or []
-        for e in entries if isinstance(entries, list) else [entries]:  # one record per launch shape
-            if (e.get("launch") == launch and e.get("kernel_source_sha") == kernel_source_sha()
-                    and e.get("ordering", "morton") == ordering):
+        for e in entries if isinstance(entries, list) else [entries]:
+            if e.get("kernel_source_sha") == kernel_source_sha() and e.get("ordering", "morton") == ordering:
                 return e["bytes_per_launch"], e.get("scaled_from")
     except Exception:
         pass

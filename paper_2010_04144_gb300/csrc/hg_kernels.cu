@@ -11,15 +11,16 @@
 //                      fused streaming + boundary rules + LBGK collision for
 //                      every site of one domain, or of many through a tile
 //                      table; A/B pull or AA in place; FP32 / FP16 / BF16
-//                      storage.  HBM-bound.
+//                      storage; run-encoded or 18-row neighbours.
+//   k_steps (hg_steps.cu) many steps of a small set of domains in one launch.
 //   k_guo_force        body force on the sites next to forced arterial outlets
 //                      (alternating coupling exchanges only).
 //   k_iolet_update     per iolet: FP64 mean of u.n and drho over its adjacent
 //                      sites (fixed order), then the boundary values of the
 //                      next step (pulse, coupled factor x source mean, or the
-//                      reverse exchange's outlet force).  It lets the next
-//                      step's stream-collide start early (programmatic
-//                      dependent launch).
+//                      reverse exchange's outlet force).  It launches while
+//                      its step's stream-collide drains and lets the next
+//                      step's start early (programmatic dependent launch).
 //   k_advance_list     bumps the per-domain completed-step counters.
 //   k_macroscopic / k_export_state / k_import_state / k_mass*: read-back.
 //
