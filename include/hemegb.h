@@ -84,6 +84,7 @@ extern "C" {
 /* ---- host-side fault injection (hg_ctx_inject_fault) ---- */
 #define HG_FAULT_ALLOC 1       /* the arg-th device allocation from now on fails (0 cancels) */
 #define HG_FAULT_DEVICE_WAIT 2 /* set the device error word as a bounded wait that gave up does */
+#define HG_FAULT_LAUNCH 3      /* the arg-th resident launch from now on is refused (0 cancels) */
 
 /* Coupling exchange direction (Section 3 alternates forward and reverse). */
 #define HG_COUPLE_FORWARD 0   /* forward after every step (default) */
@@ -306,7 +307,9 @@ int hg_coupling_factors(const int64_t *art_centres, const double *art_areas, int
  * boundary values of time t+1 (pulses; coupled inlets from the means).
  * Groups of steps run as captured CUDA graphs; the steps of a small set of
  * domains (up to 700,000 sites A/B, 450,000 AA, forward coupling) run in
- * resident launches of up to 1024 steps, with the same bits.  Asynchronous.
+ * resident launches of up to 1024 steps, with the same bits.  Where such a launch
+ * cannot be had (no memory for its tables, or the device refuses its grid, as on a
+ * stream restricted to some of the SMs) they run as the others do.  Asynchronous.
  * Passage: Section 2 (the LB step: D3Q19 streaming, LBGK collision, walls,
  * iolets) and Section 2.3 (coupled values exchanged every step). */
 int hg_step(hg_ctx *ctx, int64_t n_steps);
@@ -414,7 +417,10 @@ int hg_read_adjacent_moments(hg_domain *d, int64_t *sites_out, float *mom_out);
  * makes it returns HG_ERR_OOM and releases what it had set up; arg = 0 cancels.
  * HG_FAULT_DEVICE_WAIT: writes code arg (0 -> 1) to the context's device error
  * word, stream-ordered, exactly as a bounded device wait that gave up would;
- * the next hg_sync returns HG_ERR_TIMEOUT.  Errors: HG_ERR_ARG, HG_ERR_CUDA.
+ * the next hg_sync returns HG_ERR_TIMEOUT.
+ * HG_FAULT_LAUNCH: the arg-th resident launch (see hg_step) from now on is refused, as
+ * the device refuses one that does not fit; the set is then stepped launch by
+ * launch.  Errors: HG_ERR_ARG, HG_ERR_CUDA.
  * Passage: infrastructure: no passage (failure detection). */
 int hg_ctx_inject_fault(hg_ctx *ctx, int32_t kind, int64_t arg);
 

@@ -503,6 +503,7 @@ struct hg_ctx {
     DevBuf scratch;                 // mass partials, read-back staging
     std::atomic<int64_t> device_bytes{0};
     std::atomic<int64_t> fail_alloc_in{0};  // injected fault: the k-th next allocation fails (0 = none)
+    std::atomic<int64_t> fail_launch_in{0};  // injected fault: the k-th next resident launch is refused
     std::vector<hg_split *> splits;         // split domains (destroyed with the context)
 };
 
@@ -590,13 +591,18 @@ int fail(hg_ctx *ctx, int code, const char *fmt, ...) {
             return fail(ctx, HG_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(e_));  \
     } while (0)
 
+// Counts an injected fault down; true when this is the one to fail.
+bool fault_now(std::atomic<int64_t> &in) {
+    int64_t k = in.load();
+    while (k > 0 && !in.compare_exchange_weak(k, k - 1)) {
+    }
+    return k == 1;
+}
+
 int dev_alloc(hg_ctx *ctx, DevBuf &b, size_t bytes) {
     if (bytes == 0) bytes = 256;
     bytes = (bytes + 255) & ~(size_t)255;
-    int64_t k = ctx->fail_alloc_in.load();
-    while (k > 0 && !ctx->fail_alloc_in.compare_exchange_weak(k, k - 1)) {
-    }
-    if (k == 1) return fail(ctx, HG_ERR_OOM, "injected allocation failure (%zu bytes)", bytes);
+    if (fault_now(ctx->fail_alloc_in)) return fail(ctx, HG_ERR_OOM, "injected allocation failure (%zu bytes)", bytes);
     void *p = nullptr;
     if (ctx->alloc) {
         p = ctx->alloc(bytes, ctx->alloc_user);
@@ -1851,7 +1857,8 @@ cudaError_t steps_blocks(const hg_ctx *ctx, bool stash, int threads, size_t smem
 #undef HG_CASE
     return cudaErrorInvalidValue;
 }
-cudaError_t steps_launch(const hg_ctx *ctx, const StepsArgs &a, const StepsShape &sh) {
+cudaError_t steps_launch(hg_ctx *ctx, const StepsArgs &a, const StepsShape &sh) {
+    if (fault_now(ctx->fail_launch_in)) return cudaErrorCooperativeLaunchTooLarge;
 #define HG_CASE(S_, C_) \
     if (ctx->storage == S_ && ctx->scheme == C_) return launch_steps<S_, C_>(a, sh, ctx->stream);
     HG_CASE(0, 0) HG_CASE(0, 1) HG_CASE(1, 0) HG_CASE(1, 1) HG_CASE(2, 0) HG_CASE(2, 1)
@@ -2011,7 +2018,8 @@ int ensure_resident(hg_ctx *ctx, Plan *p) {
     return HG_OK;
 }
 
-// n steps of a plan by resident launches; `left` of them remain where it has none.
+// n steps of a plan by resident launches; `left` of them remain where it has none, or from
+// the first one that is refused on.
 int run_resident(hg_ctx *ctx, Plan *p, int64_t n, int64_t &left) {
     left = n;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -2023,7 +2031,12 @@ int run_resident(hg_ctx *ctx, Plan *p, int64_t n, int64_t &left) {
     if (rc != HG_OK || p->resident != 1) return rc;
     for (; left > 0; left -= p->res_args.n_steps) {
         p->res_args.n_steps = (int32_t)std::min<int64_t>(left, kStepsMax);
-        CU(ctx, steps_launch(ctx, p->res_args, p->res_shape));
+        if (steps_launch(ctx, p->res_args, p->res_shape) == cudaSuccess) continue;
+        // Refused: the shape counts on every SM of the device, the stream may have fewer.  The
+        // launches that take its place report whatever else was wrong.
+        cudaGetLastError();
+        p->resident = -1;
+        break;
     }
     return HG_OK;
 }
@@ -2288,6 +2301,11 @@ int hg_ctx_inject_fault(hg_ctx *ctx, int32_t kind, int64_t arg) {
     if (kind == HG_FAULT_ALLOC) {
         if (arg < 0) return fail(ctx, HG_ERR_ARG, "allocation index must be >= 0");
         ctx->fail_alloc_in = arg;
+        return HG_OK;
+    }
+    if (kind == HG_FAULT_LAUNCH) {
+        if (arg < 0) return fail(ctx, HG_ERR_ARG, "launch index must be >= 0");
+        ctx->fail_launch_in = arg;
         return HG_OK;
     }
     if (kind == HG_FAULT_DEVICE_WAIT) {
