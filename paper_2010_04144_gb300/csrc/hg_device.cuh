@@ -854,7 +854,7 @@ __device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileD
 }
 
 // A launch that started early ends only after the one before it has ended (the last block
-// waits), so that whatever follows the last of a chain follows all of it.
+// waits), so that the iolet update, a plain launch after the last of a chain, follows all of it.
 __device__ __forceinline__ void end_after_previous() {
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) wait_for_iolet_update();
 }
@@ -871,7 +871,6 @@ __global__ void __launch_bounds__(sc_threads(S, SCHEME, PAR, RUNS), sc_blocks(S,
     __shared__ DomDev D;
     __shared__ int64_t t_now;
     extern __shared__ __align__(128) int32_t stash[];
-    asm volatile("griddepcontrol.launch_dependents;");  // the iolet update may wait on this grid resident
     const TileDev tl = tiles[blockIdx.x];
     if (threadIdx.x < kWords)
         reinterpret_cast<uint64_t *>(&D)[threadIdx.x] =
@@ -892,9 +891,9 @@ __global__ void __launch_bounds__(sc_threads(S, SCHEME, PAR, RUNS), sc_blocks(S,
 template <int S, int SCHEME, int PAR, bool RUNS>
 __global__ void __launch_bounds__(sc_threads(S, SCHEME, PAR, RUNS), sc_blocks(S, SCHEME, PAR, RUNS))
     k_stream_collide_one(const __grid_constant__ DomDev D, int64_t n, int off) {
-    // a launch chained after this one (the next domain of a per-domain launch sequence, or
-    // the iolet update, which waits for this grid) may be scheduled once every block here has
-    // started; kernels launched without programmatic serialisation ignore the trigger
+    // a launch chained after this one (the next domain of a per-domain launch
+    // sequence) may be scheduled once every block here has started; kernels launched
+    // without programmatic serialisation ignore the trigger
     asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ __align__(128) int32_t stash[];
     const int64_t ts = (int64_t)sc_spt(S, SCHEME, PAR, RUNS) * blockDim.x;

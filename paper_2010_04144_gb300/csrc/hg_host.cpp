@@ -1819,8 +1819,7 @@ cudaError_t enqueue_steps(hg_ctx *ctx, Plan *p, int64_t k, int mode) {
         e = enqueue_halo(ctx, p, (int)off);
         if (e != cudaSuccess) return e;
         e = launch_iolet_update((const IoDev *)p->ios.p, p->n_ios, (const int2 *)p->chunks.p, p->n_chunks,
-                                (double2 *)p->partials.p, (unsigned *)p->counters.p, (int)off,
-                                p->n_fslots == 0 && p->n_halo == 0, ctx->stream);
+                                (double2 *)p->partials.p, (unsigned *)p->counters.p, (int)off, ctx->stream);
         if (e != cudaSuccess) return e;
     }
     return launch_advance_list((int64_t *)ctx->steps.p, (const int32_t *)p->adv.p, (int)p->doms.size(), k,
@@ -2132,7 +2131,7 @@ int hg_step_profiled(hg_ctx *ctx, int64_t n, double *ms_sc, double *ms_io, float
                                  (const int2 *)p->fslots.p, p->n_fslots, (int)j, ctx->stream);
         if (e == cudaSuccess)
             e = launch_iolet_update((const IoDev *)p->ios.p, p->n_ios, (const int2 *)p->chunks.p, p->n_chunks,
-                                    (double2 *)p->partials.p, (unsigned *)p->counters.p, (int)j, false, ctx->stream);
+                                    (double2 *)p->partials.p, (unsigned *)p->counters.p, (int)j, ctx->stream);
         cudaEventRecord(ev[3 * j + 2], ctx->stream);
     }
     if (e == cudaSuccess)

@@ -159,10 +159,8 @@ HG_SC_PART_DECL(2, 0, 2) HG_SC_PART_DECL(2, 1, 0) HG_SC_PART_DECL(2, 1, 1) HG_SC
 #undef HG_SC_PART_DECL
 // One CTA per (iolet, chunk) in `chunks`; partials: 2 doubles per chunk;
 // counters: n_ios + 1 zeroed unsigned ints (left zeroed on return).
-// early: the launch directly follows a stream-collide launch and may start before that ends
-// (programmatic dependent launch; the kernel waits for it before it reads any moments).
 cudaError_t launch_iolet_update(const IoDev *ios, int n_ios, const int2 *chunks, int n_chunks,
-                                double2 *partials, unsigned *counters, int off, bool early, cudaStream_t st);
+                                double2 *partials, unsigned *counters, int off, cudaStream_t st);
 cudaError_t launch_advance_list(int64_t *steps_base, const int32_t *idx, int n, int64_t by,
                                 cudaStream_t st);
 // Body force on the listed boundary slots ((domain, slot) pairs), right after the

@@ -18,9 +18,9 @@
 //   k_iolet_update     per iolet: FP64 mean of u.n and drho over its adjacent
 //                      sites (fixed order), then the boundary values of the
 //                      next step (pulse, coupled factor x source mean, or the
-//                      reverse exchange's outlet force).  It launches while
-//                      its step's stream-collide drains and lets the next
-//                      step's start early (programmatic dependent launch).
+//                      reverse exchange's outlet force).  It lets the next
+//                      step's stream-collide start early (programmatic
+//                      dependent launch).
 //   k_advance_list     bumps the per-domain completed-step counters.
 //   k_macroscopic / k_export_state / k_import_state / k_mass*: read-back.
 //
@@ -68,18 +68,17 @@ __global__ void __launch_bounds__(kIoChunk) k_iolet_update(const IoDev *__restri
                                                            const int2 *__restrict__ chunks,
                                                            double2 *partials, unsigned *counters,
                                                            int off) {
+    // the next step's stream-collide may launch now: it waits for this grid
+    // only where it needs the boundary values this grid produces
+    asm volatile("griddepcontrol.launch_dependents;");
     __shared__ int s_last;
     const int2 ck = chunks[blockIdx.x];
     const IoDev &I = ios[ck.x];
-    const int j = ck.y * kIoChunk + threadIdx.x;
-    const int32_t slot = j < I.n_slots ? __ldg(I.slots + j) : -1;
-    // launched while the stream-collide of this step drains: its moments from here on.  Only
-    // then may the next step's stream-collide launch; it waits for this grid only where it
-    // needs the boundary values this grid produces.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
     double su = 0.0, sr = 0.0;
-    if (slot >= 0) iolet_terms(I, I.bnd[slot], su, sr);
+    const int j = ck.y * kIoChunk + threadIdx.x;
+    if (j < I.n_slots) {
+        iolet_terms(I, I.bnd[__ldg(I.slots + j)], su, sr);
+    }
     block_sum2(su, sr);
     if (threadIdx.x == 0) {
         partials[I.part0 + ck.y] = make_double2(su, sr);
@@ -487,18 +486,10 @@ cudaError_t launch_stream_collide(const CollideCfg &cfg, const DomDev *doms, con
 }
 
 cudaError_t launch_iolet_update(const IoDev *ios, int n_ios, const int2 *chunks, int n_chunks,
-                                double2 *partials, unsigned *counters, int off, bool early, cudaStream_t st) {
+                                double2 *partials, unsigned *counters, int off, cudaStream_t st) {
     if (n_ios <= 0 || n_chunks <= 0) return cudaSuccess;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)n_chunks);
-    lc.blockDim = dim3(kIoChunk);
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, k_iolet_update, ios, n_ios, chunks, partials, counters, off);
+    k_iolet_update<<<n_chunks, kIoChunk, 0, st>>>(ios, n_ios, chunks, partials, counters, off);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_advance_list(int64_t *steps_base, const int32_t *idx, int n, int64_t by,
