@@ -307,8 +307,9 @@ int hg_coupling_factors(const int64_t *art_centres, const double *art_areas, int
  * boundary values of time t+1 (pulses; coupled inlets from the means).
  * Groups of steps run as captured CUDA graphs; the steps of a small set of
  * domains (up to 700,000 sites A/B, 450,000 AA, forward coupling) run in
- * resident launches of up to 1024 steps, with the same bits.  Where such a launch
- * cannot be had (no memory for its tables, or the device refuses its grid, as on a
+ * resident launches of up to 1024 steps, with the same bits, unless the set's
+ * iolets are so wide or many, or n_steps so few, that they would take longer.
+ * Where such a launch cannot be had (no memory for its tables, or the device refuses its grid, as on a
  * stream restricted to some of the SMs) they run as the others do.  Asynchronous.
  * Passage: Section 2 (the LB step: D3Q19 streaming, LBGK collision, walls,
  * iolets) and Section 2.3 (coupled values exchanged every step). */

@@ -444,6 +444,13 @@ struct PlanKey {
     bool operator<(const PlanKey &o) const { return doms < o.doms; }
 };
 
+// What resident_pays weighs, in us: a launched step, a step of the site blocks, and one pass of
+// the fullest iolet block over its iolets, which it has `trail` steps to make.
+struct StepsCost {
+    double launched = 0.0, launched_once = 0.0, sites = 0.0, iolets = 0.0;
+    int trail = 1;
+};
+
 struct Plan {
     std::vector<int32_t> doms;
     DevBuf tiles, ios, adv, chunks, partials, counters, rev, fslots;
@@ -467,9 +474,11 @@ struct Plan {
     int n_fslots = 0;  // (domain, slot) pairs the body-force pass visits
     int n_ios = 0;
     int n_chunks = 0;
-    // resident multi-step launches (hg_steps.cu): tables and buffers of the set, made
-    // on first use; 0 = not looked at yet, 1 = ready, -1 = the set is stepped launch by launch
+    // resident multi-step launches (hg_steps.cu): tables and buffers of the set, made on first
+    // use; 0 = not looked at yet, 1 = shape and cost known, 2 = ready, -1 = the set is stepped
+    // launch by launch
     int resident = 0;
+    StepsCost res_cost;
     DevBuf res;
     StepsArgs res_args{};
     StepsShape res_shape;
@@ -1866,11 +1875,47 @@ cudaError_t steps_launch(hg_ctx *ctx, const StepsArgs &a, const StepsShape &sh) 
 }
 
 // Largest set (sites of all its domains) that is stepped by resident launches.  Time per step of
-// a tree of n sites, launch by launch / resident (us, Morton; rows): 290k FP32 A/B 17.1 / 8.9;
-// 18.0 / 8.7, FP16 AA 16.5 / 10.5; 16.9 / 8.6; 385k FP32 A/B 19.7 / 10.6; 18.6 / 9.8, FP16 AA
-// 17.8 / 14.7; 16.7 / 11.3; 480k FP16 AA 18.6 / 18.8; 17.5 / 17.5, FP32 AA 20.7 / 20.7; 18.4 /
-// 18.0; 630k FP32 A/B 27.1 / 25.9; 22.6 / 17.8, FP16 A/B 21.7 / 15.3; 19.4 / 13.9.
+// a tree of n sites, launch by launch / resident (us, Morton; rows): 293k FP32 A/B 14.6 / 9.3;
+// 15.2 / 8.4, FP16 AA 15.0 / 10.9; 14.6 / 8.6; 441k FP32 A/B 20.8 / 14.1; 17.4 / 11.4, FP32 AA
+// 20.0 / 18.7; 16.8 / 12.6, FP16 AA 17.6 / 18.5; 16.0 / 12.2; 563k FP32 A/B 25.0 / 23.8; 19.8 /
+// 13.9; 697k FP32 A/B 29.9 / 28.7; 24.3 / 21.4, FP16 A/B 23.9 / 19.0; 16.7 / 15.2.  AA in Morton
+// order crosses just below its limit; A/B does not below its own, and nothing was measured above.
 int64_t resident_sites(const hg_ctx *ctx) { return ctx->scheme == HG_SCHEME_AB ? 700000 : 450000; }
+
+// Whether resident launches take n steps of a set no longer than launches per step do.  Each
+// iolet is summed by one block (FP64, 0.2 us per 32 slots in a full block), where the launched
+// update spreads its chunks over the card: few slots hide behind the sites, many do not.  us per
+// step, launched / resident, 100 steps a call: tube of radius 40 (5,027 slots an iolet) 50k FP32
+// A/B 13.8 / 10.9, radius 60 452k 22.1 / 25.2, radius 100 377k 28.2 / 72.0, 100 tubes in one
+// domain (200 iolets) 12.4 / 29.1, 60 packed ones (120) 12.7 / 17.7.  A call's last step also
+// waits for its own means: 1 step a call, radius 25 20k 19.6 / 27.9, radius 40 50k 21.7 / 41.5,
+// radius 6 4.5k 19.6 / 14.5, tree 166k 23.7 / 20.6, 697k 49.5 / 49.3; 4 steps a call, radius 25
+// 14.6 / 11.4, radius 40 16.3 / 18.4.  The fits below keep to these within 15 %.
+bool resident_pays(const StepsCost &c, int64_t n) {
+    const double later = std::max(c.sites, c.iolets / c.trail);
+    return c.sites + c.iolets + (double)(n - 1) * later <= (double)n * c.launched + c.launched_once;
+}
+StepsCost steps_cost(const std::vector<hg_domain *> &doms, const StepsShape &sh, int n_sets, bool coupled) {
+    StepsCost c;
+    int64_t sites = 0, slots = 0, n_ios = 0;
+    std::vector<double> block((size_t)std::max(1, n_sets), 0.0);  // iolet k of the set: block k mod n_sets
+    const double per_warp = 0.18 + 0.3 / (sh.threads / 32);       // of 32 slots; chunks count whole
+    for (const hg_domain *d : doms) {
+        sites += d->n;
+        for (int k = 0; k < d->nio; ++k) {
+            const int64_t n = d->io_ptr[k + 1] - d->io_ptr[k];
+            slots += n;
+            block[(size_t)(n_ios++ % (int64_t)block.size())] +=
+                2.0 + per_warp * (kIoChunk / 32) * (double)std::max<int64_t>(1, (n + kIoChunk - 1) / kIoChunk);
+        }
+    }
+    c.launched = 11.0 + 12e-6 * (double)sites + 2e-4 * (double)slots + 5e-3 * (double)n_ios;
+    c.launched_once = 15e-6 * (double)sites;
+    c.sites = 2.5 + 25e-6 * (double)sites;
+    if (n_ios > 0) c.iolets = *std::max_element(block.begin(), block.end());
+    c.trail = coupled ? 1 : sh.groups;  // coupled inlets wait for the means of the step before
+    return c;
+}
 
 // The shape of a resident launch over domains of the given sizes; false: none fits.  Fewest
 // tiles per block, links in shared memory if they fit, then the block size that leaves the
@@ -1880,7 +1925,8 @@ int64_t resident_sites(const hg_ctx *ctx) { return ctx->scheme == HG_SCHEME_AB ?
 // per SM 13.3 us, at two of 512 11.2).  A/B blocks of three and more tiles read their links
 // from memory (385k sites FP32 Morton: 10.6 us against 14.2 from shared memory, where only 27
 // warps per SM fit; AA the other way, 17.8 against 16.0).
-bool steps_shape(const hg_ctx *ctx, const std::vector<int64_t> &sizes, int n_ios, StepsShape &sh, int &n_site_blocks) {
+bool steps_shape(const hg_ctx *ctx, const std::vector<int64_t> &sizes, int n_ios, StepsShape &sh, int &n_site_blocks,
+                 int &n_sets) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return false;
     // iolet blocks: up to a sixth of the SMs' worth, one iolet each where that is enough, and
@@ -1908,6 +1954,7 @@ bool steps_shape(const hg_ctx *ctx, const std::vector<int64_t> &sizes, int n_ios
                     if (per_sm > room) continue;
                     best = load;
                     n_site_blocks = (int)blocks;
+                    n_sets = sets;
                     sh.threads = threads;
                     sh.smem = smem;
                     sh.stash = stash;
@@ -1919,28 +1966,43 @@ bool steps_shape(const hg_ctx *ctx, const std::vector<int64_t> &sizes, int n_ios
     return false;
 }
 
-// Tables of a resident launch; leaves p->resident at 1, or -1 where the set does not qualify.
-int ensure_resident(hg_ctx *ctx, Plan *p) {
-    if (p->resident != 0) return HG_OK;
+// Shape and cost of the set's resident launches: p->resident 0 -> 1, or -1 where it has none.
+void shape_resident(hg_ctx *ctx, Plan *p) {
     p->resident = -1;
-    if (ctx->couple_mode != HG_COUPLE_FORWARD || p->n_fslots > 0 || p->n_halo > 0) return HG_OK;
+    if (ctx->couple_mode != HG_COUPLE_FORWARD || p->n_fslots > 0 || p->n_halo > 0) return;
     std::vector<hg_domain *> doms;
     std::vector<int64_t> sizes;
     int64_t total = 0;
-    std::map<int32_t, int32_t> at;  // context index -> place in the set
+    bool coupled = false;
     for (int32_t di : p->doms) {
         hg_domain *d = di < (int32_t)ctx->doms.size() ? ctx->doms[di] : nullptr;
-        if (!d) return HG_OK;  // a split's partitions
-        at[di] = (int32_t)doms.size();
+        if (!d) return;  // a split's partitions
         doms.push_back(d);
         sizes.push_back(d->n);
         total += d->n;
-        if (19 * d->np > INT32_MAX) return HG_OK;  // links are 32-bit element indices
+        if (19 * d->np > INT32_MAX) return;  // links are 32-bit element indices
+        std::lock_guard<std::mutex> lk(ctx->mu);
+        for (const auto &c : ctx->coupled) coupled = coupled || c.first.first == di;
     }
-    if (total == 0 || total > resident_sites(ctx)) return HG_OK;
-    StepsShape sh;
-    int n_site_blocks = 0;
-    if (!steps_shape(ctx, sizes, p->n_ios, sh, n_site_blocks)) return HG_OK;
+    if (total == 0 || total > resident_sites(ctx)) return;
+    int n_site_blocks = 0, n_sets = 0;
+    if (!steps_shape(ctx, sizes, p->n_ios, p->res_shape, n_site_blocks, n_sets)) return;
+    p->res_cost = steps_cost(doms, p->res_shape, n_sets, coupled);
+    p->res_args.n_site_blocks = n_site_blocks;
+    p->resident = 1;
+}
+
+// Tables of the set's resident launches: p->resident 1 -> 2, or -1 where they cannot be had.
+int ensure_resident(hg_ctx *ctx, Plan *p) {
+    if (p->resident != 1) return HG_OK;
+    p->resident = -1;
+    const StepsShape &sh = p->res_shape;
+    std::vector<hg_domain *> doms;
+    std::map<int32_t, int32_t> at;  // context index -> place in the set
+    for (int32_t di : p->doms) {
+        at[di] = (int32_t)doms.size();
+        doms.push_back(ctx->doms[di]);
+    }
     std::vector<StepsDom> sd(doms.size());
     std::vector<TileDev> tiles;
     std::vector<StepsIo> sios;
@@ -2009,16 +2071,14 @@ int ensure_resident(hg_ctx *ctx, Plan *p) {
     a.n_tiles = (int32_t)tiles.size();
     a.n_ios = p->n_ios;
     a.n_sources = n_sources;
-    a.n_site_blocks = n_site_blocks;
     a.n_groups = sh.groups;
     a.stash_words = (int32_t)(sh.smem / 4);
-    p->res_shape = sh;
-    p->resident = 1;
+    p->resident = 2;
     return HG_OK;
 }
 
-// n steps of a plan by resident launches; `left` of them remain where it has none, or from
-// the first one that is refused on.
+// n steps of a plan by resident launches; `left` of them remain where it has none, where they
+// would take longer, or from the first one that is refused on.
 int run_resident(hg_ctx *ctx, Plan *p, int64_t n, int64_t &left) {
     left = n;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -2026,8 +2086,10 @@ int run_resident(hg_ctx *ctx, Plan *p, int64_t n, int64_t &left) {
         cudaGetLastError();
         return HG_OK;  // a caller's capture records plain launches
     }
+    if (p->resident == 0) shape_resident(ctx, p);
+    if (p->resident < 0 || !resident_pays(p->res_cost, n)) return HG_OK;
     const int rc = ensure_resident(ctx, p);
-    if (rc != HG_OK || p->resident != 1) return rc;
+    if (rc != HG_OK || p->resident != 2) return rc;
     for (; left > 0; left -= p->res_args.n_steps) {
         p->res_args.n_steps = (int32_t)std::min<int64_t>(left, kStepsMax);
         if (steps_launch(ctx, p->res_args, p->res_shape) == cudaSuccess) continue;
@@ -2040,8 +2102,8 @@ int run_resident(hg_ctx *ctx, Plan *p, int64_t n, int64_t &left) {
     return HG_OK;
 }
 
-// n steps of a plan: resident launches where the set is small, else whole groups as graph
-// replays and the rest launched directly.
+// n steps of a plan: resident launches where the set is small and they pay, else whole groups
+// as graph replays and the rest launched directly.
 int run_plan(hg_ctx *ctx, Plan *p, int64_t n, int mode) {
     int64_t left = n;
     const int rc = run_resident(ctx, p, n, left);

@@ -43,3 +43,21 @@ def test_launched_steps_of_many_iolets(gpu):
         us[scheme] = _us_per_step(ctx, 100, 4)
         ctx.close()
     assert us["ab"] < 1.2 * us["aa"], us
+
+
+@pytest.mark.parametrize("geo,storage,scheme,steps", [
+    (lambda: S.cylinder(100, 12), "f32", "ab", 100),                # 31k slots an iolet: 72 us resident, 28 launched
+    (lambda: S.parallel_tubes(100, radius=3, length=12), "f16", "aa", 20),  # 200 iolets: 28 us, 14 launched
+    (lambda: S.cylinder(40, 10), "f32", "aa", 1),                   # single steps: 41 us, 22 launched
+    (lambda: S.cylinder(50, 50), "f16", "ab", 1),                   # 64 us, 26 launched
+    (lambda: S.tree(S.TreeSpec(depth=4, scale=0.5), period=100.0), "f32", "ab", 1),
+])
+def test_way_of_stepping_is_the_faster_one(gpu, geo, storage, scheme, steps):
+    """Left to itself, a set takes no longer than launch by launch."""
+    geo = geo()
+    us = {}
+    for launches in (True, False):
+        ctx = _context(gpu, geo, storage, scheme, launches)
+        us[launches] = _us_per_step(ctx, steps, max(1, 100 // steps))
+        ctx.close()
+    assert us[False] < 1.2 * us[True], us
