@@ -85,6 +85,7 @@ extern "C" {
 #define HG_FAULT_ALLOC 1       /* the arg-th device allocation from now on fails (0 cancels) */
 #define HG_FAULT_DEVICE_WAIT 2 /* set the device error word as a bounded wait that gave up does */
 #define HG_FAULT_LAUNCH 3      /* the arg-th resident launch from now on is refused (0 cancels) */
+#define HG_FAULT_WAIT_LIMIT 4  /* waits of resident launches give up after arg polls (0: the default) */
 
 /* Coupling exchange direction (Section 3 alternates forward and reverse). */
 #define HG_COUPLE_FORWARD 0   /* forward after every step (default) */
@@ -421,7 +422,12 @@ int hg_read_adjacent_moments(hg_domain *d, int64_t *sites_out, float *mom_out);
  * the next hg_sync returns HG_ERR_TIMEOUT.
  * HG_FAULT_LAUNCH: the arg-th resident launch (see hg_step) from now on is refused, as
  * the device refuses one that does not fit; the set is then stepped launch by
- * launch.  Errors: HG_ERR_ARG, HG_ERR_CUDA.
+ * launch.
+ * HG_FAULT_WAIT_LIMIT: the bounded device waits of the resident launches made from
+ * now on give up after arg polls (at most the default, about 4 million; 0 restores
+ * it).  A launch in which one gives up ends in order, the next hg_sync returns
+ * HG_ERR_TIMEOUT, and the states of the set are not to be trusted until loaded
+ * again.  Errors: HG_ERR_ARG, HG_ERR_CUDA.
  * Passage: infrastructure: no passage (failure detection). */
 int hg_ctx_inject_fault(hg_ctx *ctx, int32_t kind, int64_t arg);
 

@@ -513,6 +513,7 @@ struct hg_ctx {
     std::atomic<int64_t> device_bytes{0};
     std::atomic<int64_t> fail_alloc_in{0};  // injected fault: the k-th next allocation fails (0 = none)
     std::atomic<int64_t> fail_launch_in{0};  // injected fault: the k-th next resident launch is refused
+    std::atomic<int64_t> wait_limit{kWaitLimit};  // polls of a resident launch's waits (fewer: injected fault)
     std::vector<hg_split *> splits;         // split domains (destroyed with the context)
 };
 
@@ -2092,6 +2093,7 @@ int run_resident(hg_ctx *ctx, Plan *p, int64_t n, int64_t &left) {
     if (rc != HG_OK || p->resident != 2) return rc;
     for (; left > 0; left -= p->res_args.n_steps) {
         p->res_args.n_steps = (int32_t)std::min<int64_t>(left, kStepsMax);
+        p->res_args.wait_limit = (uint32_t)ctx->wait_limit;
         if (steps_launch(ctx, p->res_args, p->res_shape) == cudaSuccess) continue;
         // Refused: the shape counts on every SM of the device, the stream may have fewer.  The
         // launches that take its place report whatever else was wrong.
@@ -2367,6 +2369,11 @@ int hg_ctx_inject_fault(hg_ctx *ctx, int32_t kind, int64_t arg) {
     if (kind == HG_FAULT_LAUNCH) {
         if (arg < 0) return fail(ctx, HG_ERR_ARG, "launch index must be >= 0");
         ctx->fail_launch_in = arg;
+        return HG_OK;
+    }
+    if (kind == HG_FAULT_WAIT_LIMIT) {
+        if (arg < 0 || arg > kWaitLimit) return fail(ctx, HG_ERR_ARG, "wait limit out of range");
+        ctx->wait_limit = arg ? arg : kWaitLimit;
         return HG_OK;
     }
     if (kind == HG_FAULT_DEVICE_WAIT) {

@@ -5,7 +5,7 @@
 
 namespace hg {
 
-constexpr uint32_t kWaitLimit = 1u << 22;  // polls after which a wait gives up (seconds)
+constexpr uint32_t kWaitLimit = 1u << 22;  // polls after which a wait gives up (seconds), unless a test sets fewer
 constexpr int kStepsThreads = 512;  // most threads per block
 constexpr int kStepsPerSm = 3;      // blocks of that size per SM (links in shared memory: 40 registers; else 2)
 constexpr int kStepsTiles = 8;      // most tiles a site block owns
@@ -54,6 +54,7 @@ struct StepsArgs {
     int32_t n_doms, n_tiles, n_ios, n_sources, n_site_blocks, n_steps;
     int32_t n_groups;     // iolet blocks that take the same iolets' steps in turn
     int32_t stash_words;  // dynamic shared memory of a block
+    uint32_t wait_limit;  // kWaitLimit
 };
 struct StepsShape {
     int grid = 0, threads = 0, groups = 1;

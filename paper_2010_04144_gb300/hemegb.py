@@ -24,7 +24,7 @@ SCHEME = {"ab": 0, "aa": 1}
 COUPLE = {"forward": 0, "alternate": 1}
 ORDER = {"morton": 0, "rows": 1, "bricks": 2}
 EXCHANGE = {"direct": 0, "staged": 1}
-FAULT_ALLOC, FAULT_DEVICE_WAIT, FAULT_LAUNCH = 1, 2, 3
+FAULT_ALLOC, FAULT_DEVICE_WAIT, FAULT_LAUNCH, FAULT_WAIT_LIMIT = 1, 2, 3, 4
 STORE_DTYPE = {0: np.float32, 1: np.float16, 2: None}  # bf16 is returned as uint16 bits
 
 
@@ -288,7 +288,8 @@ class Context:
     def inject_fault(self, kind, arg=0):
         """Host-side fault injection (FAULT_ALLOC: the arg-th next allocation fails;
         FAULT_DEVICE_WAIT: the device error word is set, hg_sync then reports a timeout;
-        FAULT_LAUNCH: the arg-th next resident launch is refused)."""
+        FAULT_LAUNCH: the arg-th next resident launch is refused; FAULT_WAIT_LIMIT: waits of
+        resident launches give up after arg polls, 0 restores the limit)."""
         self._ck(lib().hg_ctx_inject_fault(self.h, int(kind), int(arg)))
 
     def couple(self, src, dst, pairs):

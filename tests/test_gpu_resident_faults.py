@@ -1,5 +1,7 @@
 """Resident launches that cannot be had: the set is stepped launch by launch, with the bits of
-the resident launches.  The failures are made on the host; no GPU fault is made."""
+the resident launches.  Bounded waits in them that give up: the launch ends, hg_sync reports it,
+and the next launch is sound.  The failures are made on the host, or by a limit on the polls of a
+wait; no GPU fault is made."""
 import numpy as np
 import pytest
 
@@ -33,4 +35,48 @@ def test_refused_launch_steps_launch_by_launch(gpu, scheme, refused):
     ref = _run(gpu, scheme, calls)
     got = _run(gpu, scheme, calls, lambda ctx: ctx.inject_fault(gpu.FAULT_LAUNCH, refused))
     for a, b in zip(ref, got):
+        assert np.array_equal(a, b)
+
+
+def _coupled(gpu, scheme):
+    from paper_2010_04144_gb300 import serve
+
+    art, ven = (S.tree(S.TreeSpec(depth=3, scale=0.35), venous=v, period=37.0) for v in (False, True))
+    pairs = serve.coupled_job_from_trees(0, 0.0, 1, art, ven, [0.3] * len(ven.iolets)).pairs
+    ctx = gpu.Context(storage="f32", scheme=scheme)
+    doms = [ctx.domain(g.xyz, g.iolets) for g in (art, ven)]
+    ctx.couple(doms[0], doms[1], pairs)
+    ctx.step(10)
+    return ctx, doms
+
+
+@pytest.mark.parametrize("scheme", ["ab", "aa"])
+@pytest.mark.parametrize("polls", [1, 2, 3])
+def test_waits_that_give_up(gpu, scheme, polls):
+    """Every wait of a coupled set's launch (the step barrier, the coupled values, the iolet
+    blocks' wait) runs out after a few polls, three launches in a row; after the states are loaded
+    again the set steps to the bits of an undisturbed one."""
+    got = []
+    for disturbed in (False, True):
+        ctx, doms = _coupled(gpu, scheme)
+        saved = [d.save_state() for d in doms]
+        if disturbed:
+            ctx.inject_fault(gpu.FAULT_WAIT_LIMIT, polls)
+            ctx.step(2100)
+            with pytest.raises(gpu.HgError) as e:
+                ctx.sync()
+            assert e.value.code == gpu.HG_ERR_TIMEOUT
+            assert [d.step for d in doms] == [2110, 2110]
+            ctx.sync()  # reported once
+            ctx.inject_fault(gpu.FAULT_WAIT_LIMIT, 0)
+            for d, s in zip(doms, saved):
+                d.load_state(s)
+        ctx.step(57)
+        ctx.sync()
+        out = []
+        for d in doms:
+            out += [d.state().copy(), d.iolet_stats(), d.boundary_values(), *d.adjacent_moments(), d.step]
+        got.append(out)
+        ctx.close()
+    for a, b in zip(*got):
         assert np.array_equal(a, b)
