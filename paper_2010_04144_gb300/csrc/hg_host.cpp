@@ -630,6 +630,16 @@ int dev_alloc(hg_ctx *ctx, DevBuf &b, size_t bytes) {
     return HG_OK;
 }
 
+// An allocation whose failure the caller gets round: hg_last_error stays what it was.
+bool try_alloc(hg_ctx *ctx, DevBuf &b, size_t bytes) {
+    const hg_ctx *err_ctx = t_err_ctx;
+    std::string err = t_err;
+    if (dev_alloc(ctx, b, bytes) == HG_OK) return true;
+    t_err_ctx = err_ctx;
+    t_err = std::move(err);
+    return false;
+}
+
 void dev_free(hg_ctx *ctx, DevBuf &b) {
     if (!b.p) return;
     if (ctx->free_fn) ctx->free_fn(b.p, b.bytes, ctx->alloc_user);
@@ -2043,10 +2053,7 @@ int ensure_resident(hg_ctx *ctx, Plan *p) {
                  b_tile = pad(tiles.size() * sizeof(TileDev)), b_io = pad(sios.size() * sizeof(StepsIo)),
                  b_fed = pad(fed.size() * sizeof(StepsFed));
     const size_t b_tab = b_sync + b_dom + b_tile + b_io + b_fed;
-    if (dev_alloc(ctx, p->res, b_tab + alt) != HG_OK) {
-        cudaGetLastError();
-        return HG_OK;  // no room: launch by launch
-    }
+    if (!try_alloc(ctx, p->res, b_tab + alt)) return HG_OK;  // no room: launch by launch
     char *base = (char *)p->res.p;
     for (StepsDom &d : sd) {
         d.values = (float *)(base + b_tab + (size_t)d.values);

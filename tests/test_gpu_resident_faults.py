@@ -10,7 +10,7 @@ from paper_2010_04144_gb300 import synth as S
 pytestmark = pytest.mark.gpu
 
 
-def _run(gpu, scheme, calls, prepare=lambda ctx: None):
+def _run(gpu, scheme, calls, prepare=lambda ctx: None, after=lambda ctx: None):
     geos = [S.cylinder(radius=4, length=30, inlet=dict(kind=S.VELOCITY, value=0.02, pulse=S.PULSE_SINE, period=41.0)),
             S.tree(S.TreeSpec(depth=3, scale=0.25), period=37.0)]
     ctx = gpu.Context(storage="f32", scheme=scheme)
@@ -19,6 +19,7 @@ def _run(gpu, scheme, calls, prepare=lambda ctx: None):
     for n in calls:
         ctx.step(n)
     ctx.sync()
+    after(ctx)
     out = []
     for d in doms:
         out += [d.state().copy(), d.iolet_stats(), d.boundary_values(), *d.adjacent_moments(), d.step]
@@ -34,6 +35,18 @@ def test_refused_launch_steps_launch_by_launch(gpu, scheme, refused):
     calls = (2051, 37, 3)
     ref = _run(gpu, scheme, calls)
     got = _run(gpu, scheme, calls, lambda ctx: ctx.inject_fault(gpu.FAULT_LAUNCH, refused))
+    for a, b in zip(ref, got):
+        assert np.array_equal(a, b)
+
+
+def test_no_memory_for_tables(gpu):
+    """The plan's eight buffers are had, the resident tables are not: the set is stepped launch by
+    launch, and the call that returned HG_OK leaves no error text behind."""
+    errors = []
+    ref = _run(gpu, "ab", (37, 3))
+    got = _run(gpu, "ab", (37, 3), lambda ctx: ctx.inject_fault(gpu.FAULT_ALLOC, 9),
+               lambda ctx: errors.append(gpu.lib().hg_last_error(ctx.h)))
+    assert errors == [b""]
     for a, b in zip(ref, got):
         assert np.array_equal(a, b)
 
