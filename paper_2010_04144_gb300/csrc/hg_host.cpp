@@ -510,6 +510,9 @@ struct hg_ctx {
     std::atomic<int> couple_mode{HG_COUPLE_FORWARD};  // read by builds on another thread
     std::map<PlanKey, std::unique_ptr<Plan>> plans;
     DevBuf scratch;                 // mass partials, read-back staging
+    // boundary values and moments of a resident launch's steps: one for all sets, of the largest
+    // one's size (the launches follow one another on the stream; none reads what another left)
+    DevBuf res_scratch;
     std::atomic<int64_t> device_bytes{0};
     std::atomic<int64_t> fail_alloc_in{0};  // injected fault: the k-th next allocation fails (0 = none)
     std::atomic<int64_t> fail_launch_in{0};  // injected fault: the k-th next resident launch is refused
@@ -659,6 +662,7 @@ void drop_plans(hg_ctx *ctx) {
             dev_free(ctx, *b);
     }
     ctx->plans.clear();
+    dev_free(ctx, ctx->res_scratch);
 }
 
 // Appends DomDev::io_words (one per boundary slot) to the slots' 18 link codes.
@@ -2003,6 +2007,24 @@ void shape_resident(hg_ctx *ctx, Plan *p) {
     p->resident = 1;
 }
 
+// At least `bytes` of ctx->res_scratch; `room`: whether they could be had.  The tables of the sets
+// that used a smaller one are made again when those are stepped next.
+int ensure_res_scratch(hg_ctx *ctx, size_t bytes, bool &room) {
+    room = true;
+    if (ctx->res_scratch.p && ctx->res_scratch.bytes >= bytes) return HG_OK;
+    if (ctx->res_scratch.p) {
+        CU(ctx, cudaStreamSynchronize(ctx->stream));
+        for (auto &kv : ctx->plans)
+            if (kv.second->resident == 2) {
+                dev_free(ctx, kv.second->res);
+                kv.second->resident = 1;
+            }
+        dev_free(ctx, ctx->res_scratch);
+    }
+    room = try_alloc(ctx, ctx->res_scratch, bytes);
+    return HG_OK;
+}
+
 // Tables of the set's resident launches: p->resident 1 -> 2, or -1 where they cannot be had.
 int ensure_resident(hg_ctx *ctx, Plan *p) {
     if (p->resident != 1) return HG_OK;
@@ -2053,11 +2075,13 @@ int ensure_resident(hg_ctx *ctx, Plan *p) {
                  b_tile = pad(tiles.size() * sizeof(TileDev)), b_io = pad(sios.size() * sizeof(StepsIo)),
                  b_fed = pad(fed.size() * sizeof(StepsFed));
     const size_t b_tab = b_sync + b_dom + b_tile + b_io + b_fed;
-    if (!try_alloc(ctx, p->res, b_tab + alt)) return HG_OK;  // no room: launch by launch
-    char *base = (char *)p->res.p;
+    bool room = false;
+    const int rc = ensure_res_scratch(ctx, alt, room);
+    if (rc != HG_OK || !room || !try_alloc(ctx, p->res, b_tab)) return rc;  // no room: launch by launch
+    char *base = (char *)p->res.p, *scratch = (char *)ctx->res_scratch.p;
     for (StepsDom &d : sd) {
-        d.values = (float *)(base + b_tab + (size_t)d.values);
-        d.moments = (float4 *)(base + b_tab + (size_t)d.moments);
+        d.values = (float *)(scratch + (size_t)d.values);
+        d.moments = (float4 *)(scratch + (size_t)d.moments);
     }
     std::vector<char> up(b_tab, 0);
     char *u = up.data() + b_sync;

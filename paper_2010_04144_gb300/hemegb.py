@@ -24,6 +24,8 @@ SCHEME = {"ab": 0, "aa": 1}
 COUPLE = {"forward": 0, "alternate": 1}
 ORDER = {"morton": 0, "rows": 1, "bricks": 2}
 EXCHANGE = {"direct": 0, "staged": 1}
+# most sites of a set that hg_step steps by resident launches, by scheme
+RESIDENT_SITES_AB, RESIDENT_SITES_AA = 700_000, 450_000
 FAULT_ALLOC, FAULT_DEVICE_WAIT, FAULT_LAUNCH, FAULT_WAIT_LIMIT = 1, 2, 3, 4
 STORE_DTYPE = {0: np.float32, 1: np.float16, 2: None}  # bf16 is returned as uint16 bits
 

@@ -51,7 +51,10 @@ def footprint_bytes(n_sites, storage, scheme, n_iolets=2, iolet_radii=None, reor
     built (4 bytes per site plus at most 16 bytes per site of run offsets); moments, link
     codes, link coefficients and site index per boundary slot (168 B) plus one list entry
     per (site, iolet) pair; per-iolet values; the two site permutations of a reordered
-    layout; and the 256-byte rounding of each buffer.  With the iolet radii the boundary slots are bounded per iolet
+    layout; and the 256-byte rounding of each buffer.  Then its part in stepping a set it belongs
+    to: tiles, iolet descriptors and reduction chunks of the launches, and for a domain small
+    enough for resident launches their tables, 1024 boundary values per iolet and four moments
+    per boundary slot.  With the iolet radii the boundary slots are bounded per iolet
     (adjacent_bound); without them 5% of the sites is assumed."""
     np_ = max(128, (n_sites + 127) // 128 * 128)
     copies = 2 if scheme == H.SCHEME["ab"] else 1
@@ -62,7 +65,11 @@ def footprint_bytes(n_sites, storage, scheme, n_iolets=2, iolet_radii=None, reor
         n_iolets = len(iolet_radii)
     else:
         adjacent = pairs = 0.05 * n_sites
-    return int(per_site * np_ + 168 * adjacent + 4 * pairs + 64 * n_iolets + 20 * 256 + 4 * 4096)
+    domain = per_site * np_ + 168 * adjacent + 4 * pairs + 64 * n_iolets + 20 * 256 + 4 * 4096
+    launches = 16 / 256 * np_ + (24 / 256 + 8) * pairs + 256 * n_iolets + 10 * 256
+    if n_sites <= (H.RESIDENT_SITES_AB if scheme == H.SCHEME["ab"] else H.RESIDENT_SITES_AA):
+        launches += 16 / 64 * np_ + 64 * adjacent + (4096 + 32) * n_iolets + 512 + 8 * 256
+    return int(domain + launches)
 
 
 def geometry_footprint(geo, storage, scheme, reordered=False):

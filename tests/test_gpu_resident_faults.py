@@ -93,3 +93,37 @@ def test_waits_that_give_up(gpu, scheme, polls):
         ctx.close()
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+def _live(ctx):
+    return sum(t.numel() for t in ctx._alloc.live.values())
+
+
+@pytest.mark.parametrize("storage,scheme", [("f32", "ab"), ("f16", "aa")])
+def test_device_memory_of_small_sets(gpu, storage, scheme):
+    """What domains and their stepping hold stays below the server's estimate, and sets that are
+    stepped in turn share one buffer of boundary values and moments."""
+    from paper_2010_04144_gb300 import serve
+
+    geos = [S.parallel_tubes(12, radius=4, length=20), S.cylinder(radius=9, length=30),
+            S.tree(S.TreeSpec(depth=4, scale=0.2), period=37.0)]
+    ctx = gpu.Context(storage=storage, scheme=scheme)
+    before = _live(ctx)
+    doms = [ctx.domain(g.xyz, g.iolets) for g in geos]
+    ctx.step(100)
+    ctx.sync()
+    held = _live(ctx) - before
+    assert held <= sum(serve.geometry_footprint(g, ctx.storage, ctx.scheme) for g in geos)
+    for sub in (doms[:1], doms[1:], doms[:2]):
+        ctx.step_domains(sub, 100)
+    ctx.sync()
+    # three more plans: tables (a tile of 16 bytes per 64 sites or more, descriptors), no scratch
+    tables = 3 * (sum(g.n for g in geos) / 2 + 512 * sum(len(g.iolets) for g in geos) + 32 * 256)
+    assert _live(ctx) - before - held <= tables
+    # a larger set replaces the buffer; the first set steps on with new tables
+    big = ctx.domain(*(lambda g: (g.xyz, g.iolets))(S.parallel_tubes(40, radius=3, length=12)))
+    ctx.step(100)
+    ctx.step_domains(doms, 100)
+    ctx.sync()
+    assert [d.step for d in doms + [big]] == [500, 500, 400, 100]
+    ctx.close()
