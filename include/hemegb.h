@@ -332,7 +332,8 @@ int hg_step_profiled(hg_ctx *ctx, int64_t n_steps, double *ms_stream_collide,
 
 /* Change the launch shape recorded for an existing context (threads per block:
  * multiple of 32, <= 512; sites per thread: 1, 2 or 4; kernel variant as in
- * hg_ctx_params, which says what it decides).  Results do not depend on it.
+ * hg_ctx_params, which says that it decides nothing).  Neither results nor
+ * launches depend on it, and nothing is waited for or built again.
  * Errors: HG_ERR_ARG.
  * Passage: infrastructure: no passage. */
 int hg_ctx_set_launch(hg_ctx *ctx, int32_t block_size, int32_t sites_per_thread,

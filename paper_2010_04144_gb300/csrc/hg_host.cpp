@@ -2265,13 +2265,9 @@ int hg_ctx_set_launch(hg_ctx *ctx, int32_t block, int32_t spt, int32_t variant) 
                                      "thread (AA only), 8..11 with the shapes of 3, 5, 6, 7, 12 with 1 or "
                                      "2 sites per thread (AA only), 13 with 2 or 4 sites per thread, or 14 "
                                      "with 2 sites per thread (AA only)");
-    if (block == ctx->block && spt == ctx->spt && variant == ctx->variant) return HG_OK;
-    CU(ctx, cudaSetDevice(ctx->device));
-    CU(ctx, cudaStreamSynchronize(ctx->stream));
-    ctx->block = block;
+    ctx->block = block;  // recorded; no launch depends on them
     ctx->spt = spt;
     ctx->variant = variant;
-    drop_plans(ctx);
     return HG_OK;
 }
 

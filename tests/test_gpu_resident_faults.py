@@ -127,3 +127,19 @@ def test_device_memory_of_small_sets(gpu, storage, scheme):
     ctx.sync()
     assert [d.step for d in doms + [big]] == [500, 500, 400, 100]
     ctx.close()
+
+
+def test_launch_setting_keeps_plans(gpu):
+    """A launch setting selects nothing, so setting one frees and builds nothing again."""
+    geo = S.cylinder(radius=4, length=20)
+    ctx = gpu.Context(storage="f16", scheme="aa")
+    d = ctx.domain(geo.xyz, geo.iolets)
+    ctx.step(20)
+    held = set(ctx._alloc.live)
+    for launch in ((128, 2, 14), (256, 1, 0), (128, 2, 1)):
+        ctx.set_launch(*launch)
+        assert set(ctx._alloc.live) == held
+        ctx.step(20)
+        assert set(ctx._alloc.live) == held
+    assert d.step == 80
+    ctx.close()
