@@ -38,8 +38,11 @@ FALLBACK_HBM_GBS = 6800.0
 
 # device site orderings the autotuner tries (every one gives bit-identical results)
 ORDERINGS = ("morton", "rows", "bricks")
+# threads per block, sites per thread and variant select nothing (the library picks the kernel form
+# and launch shape of every launch), so tuning is left one setting and decides the ordering
+SETTING = ((256, 1, 0),)
 
-def bytes_per_update(storage, scheme, variant=0, n=1, n_runs=0):
+def bytes_per_update(storage, scheme, n=1, n_runs=0):
     """Algorithmic bytes per site update of the stream-collide kernel: the 19 populations
     read and written once each, plus the neighbour table on pull steps (every A/B step, the
     odd AA steps): its 18 rows (72 bytes), or on a domain that has runs (the library then
@@ -54,9 +57,8 @@ def bytes_per_update(storage, scheme, variant=0, n=1, n_runs=0):
 
 def domain_bytes(ctx, storage, scheme, doms):
     """Bytes per update averaged over the domains one launch sequence steps."""
-    v = ctx.launch[2]
     tot = sum(d.n for d in doms)
-    return sum(bytes_per_update(storage, scheme, v, d.n, d.info()["n_runs"]) * d.n for d in doms) / tot
+    return sum(bytes_per_update(storage, scheme, d.n, d.info()["n_runs"]) * d.n for d in doms) / tot
 DTYPE_NAME = {"f32": "f32", "f16": "f16-stored/f32-compute", "bf16": "bf16-stored/f32-compute"}
 
 
@@ -143,7 +145,7 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def profiled_traffic(variant_key, launch, ordering="morton"):
+def profiled_traffic(variant_key, ordering="morton"):
     """DRAM bytes per launch from the committed ncu summary, if it matches this kernel build
     and site ordering (the library picks the launch shape itself)."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
@@ -212,13 +214,28 @@ def whole_job_mflups(sites_per_rank, world_size, steps, max_ms):
     return sites_per_rank * world_size * steps / (max_ms / 1e3) / 1e6
 
 
+def kernel_form(n_runs):
+    """The stream-collide kernel the library takes over a domain with that many runs."""
+    return "run-encoded table" if n_runs > 0 else "18-row table"
+
+
+def launches_of(n, steps, scheme, iolets):
+    """Kernels launched by `steps` steps of one domain of n sites (forward coupling): resident
+    launches of up to 1024 steps for a small one (trees and tubes), else a stream-collide and an
+    iolet update per step and a counter update per graph of 16."""
+    from paper_2010_04144_gb300 import hemegb as H
+
+    if n <= (H.RESIDENT_SITES_AB if scheme == "ab" else H.RESIDENT_SITES_AA):
+        return -(-steps // 1024)
+    return steps * (1 + (1 if iolets else 0)) + (steps + 15) // 16
+
+
 def time_variant(H, geo, storage, scheme, steps, warmup, dist, device, sampler, launch=None,
                  orderings=ORDERINGS, min_timed_s=MIN_TIMED_S):
-    """Autotuned (or given) site ordering and launch shape, device-timed steps (graphs),
-    per-kernel times, e2e job."""
+    """Tuned (or given) site ordering, device-timed steps (graphs), per-kernel times, e2e job."""
     import torch
 
-    from paper_2010_04144_gb300.autotune import autotune, tune_ordering
+    from paper_2010_04144_gb300.autotune import tune_ordering
 
     nvtx = torch.cuda.nvtx
     tag = f"{storage}:{scheme}"
@@ -230,7 +247,7 @@ def time_variant(H, geo, storage, scheme, steps, warmup, dist, device, sampler, 
             return c
 
         nvtx.range_push(f"{tag}-ordering")
-        ordering, _, table = tune_ordering(make, orderings)
+        ordering, _, table = tune_ordering(make, orderings, SETTING)
         order_ms = {o: round(v[1], 4) for o, v in table.items()}
         nvtx.range_pop()
     else:
@@ -240,13 +257,8 @@ def time_variant(H, geo, storage, scheme, steps, warmup, dist, device, sampler, 
         d = ctx.domain(geo.xyz, geo.iolets, tau=0.8, ordering=ordering)
         n = d.n
         st = ctx.stream
-        nvtx.range_push(f"{tag}-autotune")
-        if launch is None:
-            best, timing = autotune(ctx)
-        else:  # a fixed shape (profiling one kernel form), no tuning
+        if launch is not None:  # a given setting
             ctx.set_launch(*launch)
-            best, timing = tuple(launch), {}
-        nvtx.range_pop()
         # warm-up, then the timed regions: exactly `steps` steps each, barrier + sync on both
         # sides, repeated until MIN_TIMED_S of device time has passed; the median is reported
         ctx.step(warmup)
@@ -290,15 +302,13 @@ def time_variant(H, geo, storage, scheme, steps, warmup, dist, device, sampler, 
             raise RuntimeError("read-back failed")
         barrier(dist)
         e2e_s = max_over_ranks(time.perf_counter() - t0, dist, device)
-        gs = 16
-        launches = steps * (1 + (1 if geo.iolets else 0)) + (steps + gs - 1) // gs
+        launches = launches_of(n, steps, scheme, geo.iolets)
         n_runs = d.info()["n_runs"]
         return dict(n=n, ms=ms, reps=len(reps), timed_s=total / 1e3, ms_sc=ms_sc, ms_io=ms_io,
-                    n_runs=n_runs, bytes_per_update=bytes_per_update(storage, scheme, best[2], n, n_runs),
+                    n_runs=n_runs, bytes_per_update=bytes_per_update(storage, scheme, n, n_runs),
                     ordering=ordering, ordering_ms=order_ms, e2e_s=e2e_s, h2d=int(state.size),
                     d2h=int(n * 16), launches=launches, device_bytes=d.info()["device_bytes"],
-                    launch={"block": best[0], "sites_per_thread": best[1], "kernel_variant": best[2]},
-                    tuning_ms={f"{b}x{t}v{v}": round(x, 4) for (b, t, v), x in timing.items()})
+                    kernel=kernel_form(n_runs))
     finally:
         ctx.close()
 
@@ -408,8 +418,8 @@ def serve_requests(args, pool=None):
 
 
 def serve_tuning(args, H, device, reqs, geos):
-    """Site ordering and launch shape of the packed (tile-table) launches serving runs: tuned
-    on a context that holds the stream's first requests, as a tick would pack them."""
+    """Site ordering of the packed launches serving runs: tuned on a context that holds the
+    stream's first requests, as a tick would pack them."""
     from paper_2010_04144_gb300 import synth as S
     from paper_2010_04144_gb300.autotune import tune_ordering
 
@@ -421,7 +431,7 @@ def serve_tuning(args, H, device, reqs, geos):
             c.domain(g.xyz, g.iolets, ordering=o)
         return c
 
-    o, shape, table = tune_ordering(make, ORDERINGS if args.serve_ordering == "auto" else (args.serve_ordering,))
+    o, shape, table = tune_ordering(make, ORDERINGS if args.serve_ordering == "auto" else (args.serve_ordering,), SETTING)
     return o, shape, {k: round(v[1], 4) for k, v in table.items()}, int(sum(g.n for g in pack))
 
 
@@ -462,7 +472,7 @@ def serve_stats(args, H, device, prepared=None):
            "budget_gb": args.budget_gb, "tick_steps": 100, "tick_site_steps": args.serve_tick_sites or None,
            "scheme": args.serve_scheme,
            "storage": args.serve_storage, "ordering": ordering, "ordering_ms": order_ms,
-           "launch": list(shape), "launch_tuned_on_sites": tuned_sites,
+           "ordering_tuned_on_sites": tuned_sites,
            "build_workers": args.serve_build_workers, "policy": args.serve_policy,
            "total_sites": int(sum(sites)), "offered_mflups": offered, "geometry_generation_s": gen_s}
     return st, cfg
@@ -483,7 +493,6 @@ def run_coupled(args, H, device):
     import torch
 
     from paper_2010_04144_gb300 import synth as S
-    from paper_2010_04144_gb300.autotune import autotune
 
     from paper_2010_04144_gb300 import serve as SV
 
@@ -511,7 +520,6 @@ def run_coupled(args, H, device):
                 pairs.append((k, k, float(f[0])))
         ctx.couple(da, dv, pairs)
         ctx.set_coupling_mode(args.coupled_mode)
-        best, _ = autotune(ctx)
         # let the inlet's wave reach every outlet (and the coupled inlets) before timing
         ctx.step(args.coupled_settle)
         ctx.step(args.warmup)
@@ -565,7 +573,7 @@ def run_coupled(args, H, device):
                            "scheme": args.coupled_scheme, "exchange": args.coupled_mode,
                            "ordering": args.coupled_ordering, "n_runs": [da.info()["n_runs"], dv.info()["n_runs"]],
                            "settle_steps": args.coupled_settle,
-                           "launch": {"block": best[0], "sites_per_thread": best[1], "kernel_variant": best[2]}},
+                           "kernel": [kernel_form(x.info()["n_runs"]) for x in (da, dv)]},
                 "roofline": {"bound": "hbm", "achieved": B * n / (per / 1e3) / 1e9, "peak": peak,
                              "unit": "GB/s", "frac": B * n / (per / 1e3) / 1e9 / peak,
                              "bytes_per_update": B},
@@ -588,43 +596,26 @@ def run_split(args, H, device):
     unsplit domain's tuned ordering; results are bit-identical, so only the time differs."""
     import torch
 
-    from paper_2010_04144_gb300.autotune import autotune, autotune_split, tune_ordering
+    from paper_2010_04144_gb300.autotune import tune_ordering
 
     geo, cfg = workload(scale=args.scale)
     rows = []
-    launch = None
-    tuned = {}
     ordering = args.split_ordering
     if ordering == "auto":  # the unsplit domain's best ordering, used by every partition too
         def make(o):
             c = H.Context(device=device, storage="f32", scheme="ab")
             c.domain(geo.xyz, geo.iolets, ordering=o)
             return c
-        ordering, _, _ = tune_ordering(make, ORDERINGS)
+        ordering, _, _ = tune_ordering(make, ORDERINGS, SETTING)
     runs = [(0, None)] + [(int(x), ex) for x in args.parts.split(",") for ex in args.split_exchange.split(",")]
     for k, ex in runs:
         ctx = H.Context(device=device, storage="f32", scheme="ab")
         try:
             if k == 0:
                 obj = ctx.domain(geo.xyz, geo.iolets, ordering=ordering)
-                if args.split_launch:
-                    b, rest = args.split_launch.split("x")
-                    launch = (int(b), *[int(x) for x in rest.split("v")])
-                    ctx.set_launch(*launch)
-                else:
-                    launch, _ = autotune(ctx)
             else:
                 obj = ctx.split(geo.xyz, geo.iolets, k, boundary_weight=args.boundary_weight, ordering=ordering,
                                 exchange=ex)
-                if args.split_launch:
-                    ctx.set_launch(*launch)
-                    split_shape = launch
-                elif (k, "shape") in tuned:   # the other transport reuses the shape tuned for k
-                    split_shape = tuned[(k, "shape")]
-                    ctx.set_launch(*split_shape)
-                else:
-                    split_shape, _ = autotune_split(ctx, obj)
-                    tuned[(k, "shape")] = split_shape
             obj.step(args.warmup) if k else ctx.step(args.warmup)
             torch.cuda.synchronize()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -636,8 +627,7 @@ def run_split(args, H, device):
             halo = sum(obj.info(p)["halo_in"] for p in range(k)) if k else 0
             ghosts = sum(obj.info(p)["ghosts"] for p in range(k)) if k else 0
             rows.append({"parts": k, "exchange": ex, "ms_per_step": ms, "mflups": geo.n / (ms / 1e3) / 1e6,
-                         "halo_values_per_step": halo, "ghost_sites": ghosts,
-                         "launch": list(launch if k == 0 else split_shape)})
+                         "halo_values_per_step": halo, "ghost_sites": ghosts})
         finally:
             ctx.close()
     base = rows[0]["ms_per_step"]
@@ -648,7 +638,7 @@ def run_split(args, H, device):
             "steps": args.steps, "warmup": args.warmup, "higher_is_better": True, "dtype": "f32",
             "data": "synthetic (seeded tree geometry, rest initial state)",
             "config": {**cfg, "steps_per_job": args.steps, "storage": "f32", "scheme": "ab",
-                       "launch": list(launch), "ordering": ordering,
+                       "ordering": ordering,
                        "split": "contiguous Morton ranges, each partition's sites in the device ordering; "
                                 "halo exchange every step on one device (direct: one kernel; staged: "
                                 "pack, one copy per partition pair, unpack)",
@@ -659,7 +649,7 @@ def run_split(args, H, device):
 
 def time_large(args, H, device, geo, results):
     """The precision workload's ~77M-site tree in the 32- and 16-bit forms, each with the
-    ordering and launch shape the ~10M-site tuning chose for it: MFLUPS of the whole step
+    ordering the ~10M-site tuning chose for it: MFLUPS of the whole step
     and the stream-collide kernel's fraction of its HBM roofline."""
     import torch
 
@@ -673,8 +663,6 @@ def time_large(args, H, device, geo, results):
         ctx = H.Context(device=device, storage=storage, scheme=scheme)
         try:
             d = ctx.domain(geo.xyz, geo.iolets, ordering=r["ordering"])
-            L = r["launch"]
-            ctx.set_launch(L["block"], L["sites_per_thread"], L["kernel_variant"])
             ctx.step(args.warmup)
             torch.cuda.synchronize()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -689,7 +677,7 @@ def time_large(args, H, device, geo, results):
             out[f"{storage}:{scheme}"] = {"mflups": d.n / (ms / 1e3) / 1e6, "ms_per_step": ms,
                                           "bytes_per_update": B,
                                           "roofline_frac": B * d.n / (ms_sc / 16 / 1e3) / 1e9 / peak,
-                                          "ordering": r["ordering"], "launch": L,
+                                          "ordering": r["ordering"], "kernel": kernel_form(d.info()["n_runs"]),
                                           "device_gb": d.info()["device_bytes"] / 1e9}
         finally:
             ctx.close()
@@ -702,7 +690,6 @@ def run_precision(args, H, device):
     import torch
 
     from paper_2010_04144_gb300 import synth as S
-    from paper_2010_04144_gb300.autotune import autotune
 
     spec = S.TreeSpec(depth=8, root_radius=40.0, seed=2010041442, scale=args.precision_scale)
     geo = S.tree(spec, inlet_speed=0.05, period=1000.0)
@@ -712,7 +699,6 @@ def run_precision(args, H, device):
         ctx = H.Context(device=device, storage=storage, scheme=scheme)
         try:
             d = ctx.domain(geo.xyz, geo.iolets, ordering="rows")
-            best, _ = autotune(ctx)
             ctx.step(args.warmup)
             torch.cuda.synchronize()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -726,7 +712,7 @@ def run_precision(args, H, device):
             per = ms_sc / min(args.steps, 100)
             out[f"{storage}:{scheme}"] = {"mflups": d.n * args.steps / (ms / 1e3) / 1e6,
                                           "roofline_frac": B * d.n / (per / 1e3) / 1e9 / peak,
-                                          "launch": list(best), "device_gb": d.info()["device_bytes"] / 1e9}
+                                          "kernel": kernel_form(d.info()["n_runs"]), "device_gb": d.info()["device_bytes"] / 1e9}
         finally:
             ctx.close()
     err = {}
@@ -767,7 +753,8 @@ def main():
     ap.add_argument("--impl", default="hemegb", choices=["hemegb", "reference"])
     ap.add_argument("--scale", type=float, default=1.71)
     ap.add_argument("--variants", default="f32:ab,f32:aa,f16:ab,f16:aa,bf16:aa",
-                    help="storage:scheme list; append @BLOCKxSPTvVARIANT to fix a launch shape")
+                    help="storage:scheme list; append @BLOCKxSPTvVARIANT to set a launch "
+                         "setting (selects nothing; the ordering is then not tuned)")
     ap.add_argument("--headline", default="f32:best")
     ap.add_argument("--min-timed-s", type=float, default=MIN_TIMED_S,
                     help="device time each variant's repeated K-step measurement covers (0: three)")
@@ -778,7 +765,7 @@ def main():
                     help="split config: auto (the unsplit domain's tuned ordering) or morton / rows / bricks")
     ap.add_argument("--split-exchange", default="direct,staged",
                     help="split config: halo transports to time (direct, staged)")
-    ap.add_argument("--split-launch", default="", help="split config: fixed launch BLOCKxSPTvVARIANT (no tuning)")
+    ap.add_argument("--split-launch", default="", help="split config: launch setting (accepted, selects nothing)")
     ap.add_argument("--boundary-weight", type=float, default=1.0,
                     help="split config: load-balancing cost of a site next to an iolet")
     ap.add_argument("--coupled-scale", type=float, default=2.12)
@@ -892,14 +879,14 @@ def main():
     total_sites = h["n"] * ws
     value = whole_job_mflups(h["n"], ws, args.steps, h["ms"])
     e2e_value = total_sites * args.steps / h["e2e_s"] / 1e6
-    traffic, scaled_from = profiled_traffic(f"{head[0]}:{head[1]}", h["launch"], h["ordering"])
+    traffic, scaled_from = profiled_traffic(f"{head[0]}:{head[1]}", h["ordering"])
     line = {
         "metric": METRIC,
         "value": value, "unit": "MFLUPS", "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": h["ms"] / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": DTYPE_NAME[head[0]],
         "data": "synthetic (seeded tree geometry, rest initial state)",
-        "config": {**cfg, "storage": head[0], "scheme": head[1], "launch": h["launch"],
+        "config": {**cfg, "storage": head[0], "scheme": head[1], "kernel": h["kernel"],
                    "ordering": h["ordering"],
                    "timing": f"median of {h['reps']} back-to-back {args.steps}-step measurements "
                              f"({h['timed_s']:.2f} s of device time)",
@@ -923,8 +910,8 @@ def main():
                                    "bytes_per_update": r["bytes_per_update"], "n_runs": r["n_runs"],
                                    "stream_collide_ms": r["ms_sc"] / args.steps,
                                    "iolet_update_ms": r["ms_io"] / args.steps,
-                                   "launch": r["launch"], "ordering": r["ordering"],
-                                   "ordering_ms": r["ordering_ms"], "tuning_ms": r["tuning_ms"],
+                                   "kernel": r["kernel"], "ordering": r["ordering"],
+                                   "ordering_ms": r["ordering_ms"],
                                    "device_bytes": r["device_bytes"]}
                      for (s, c), r in results.items()},
     }
