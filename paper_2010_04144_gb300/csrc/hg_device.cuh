@@ -18,7 +18,6 @@
 namespace hg {
 namespace {
 
-
 // ---- D3Q19 (rest; +x,-x,+y,-y,+z,-z; 12 diagonals in opposite pairs) ----
 __host__ __device__ constexpr int CX(int i) {
     return (i == 1 || i == 7 || i == 9 || i == 11 || i == 13) ? 1
@@ -412,8 +411,12 @@ __device__ __forceinline__ void apply_iolet_links(const DomDev &D, const float *
 }
 // A stream-collide launch may start while the previous step's iolet update is
 // still running (programmatic dependent launch): everything it reads except the
-// boundary values was complete before that update began.  Only the sites with
-// an iolet link use those values (and overwrite the moments slot the update
+// boundary values was complete before that update began, which is a plain launch
+// behind the previous step's stream-collide.  (Launched early as well, waiting here for
+// that step, it would let this launch go on the strength of a wait that makes the
+// step's writes visible to the update alone; it gained 1.6 us of a 36 us step at 1M sites
+// and cost A/B steps of 35k sites with 200 iolets 4.5 of 12.6.)  Only the sites with
+// an iolet link use the boundary values (and overwrite the moments slot the update
 // reads), so only they wait here for the update to finish.  Without an
 // overlapping launch the wait returns at once.
 __device__ __forceinline__ void wait_for_iolet_update() {
@@ -597,7 +600,6 @@ __device__ __forceinline__ void tile_aa_even_pairs(const DomDev &D, const TileDe
     }
 }
 
-// ==== one site per thread: the A/B step and the AA odd step ====================
 // ==== one site per thread: the A/B step and the AA odd step ====================
 // FP32 AA odd through the run encoding: bound by the misaligned scatter's sectors (268 us on the
 // ~10M-site tree, 303 before the links were decoded as below); 40 registers, so 48 warps per SM
@@ -787,12 +789,12 @@ __device__ __noinline__ void tail_site(const DomDev &D, const typename St<S>::T 
                                 2 * (int)blockDim.x);
 }
 
+// One tile of one domain, after the prologue has located it.
 // PAR is the parity of the step this launch executes: 0 = even, 1 = odd (the
 // AA step kind), 2 = read from the domain's step counter per block (A/B, and AA
 // batches whose domains are at different parities).  RUNS: the domain has a run
 // encoding (the host launches the form only on such domains; a domain without one here is
 // reported through the error word, code 2, and left untouched).
-// One tile of one domain, after the prologue has located it.
 template <int S, int SCHEME, int PAR, bool RUNS>
 __device__ __forceinline__ void stream_collide_tile(const DomDev &D, const TileDev &tl, bool odd, int32_t *stash) {
     using T = typename St<S>::T;
