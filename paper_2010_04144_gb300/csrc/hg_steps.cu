@@ -7,7 +7,7 @@
 // the chain of dependent latencies in the iolet update.  Here a cooperative grid stays
 // resident for all the steps: most blocks own fixed tiles of sites and keep their links in
 // shared memory, a few blocks do the iolet work, and one grid barrier (1.4 us) ends each step.
-// Per step, launches -> resident: 4.5k sites FP32 A/B 11.4 -> 3.1 us, 13k FP32 AA 12.0 -> 2.8,
+// Per step, launches -> resident: 4.5k sites FP32 A/B 11.4 -> 2.8 us, 13k FP32 AA 12.0 -> 2.8,
 // 166k FP32 A/B 15.0 -> 6.1, 16 tubes of 279k FP16 AA 21.9 -> 11.2, coupled pair of 339k FP16
 // AA 22.9 -> 11.2.  What bounds it now: the barrier and one round of L2 latencies up to ~50k
 // sites, then L2 traffic.
